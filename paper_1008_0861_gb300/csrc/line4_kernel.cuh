@@ -78,8 +78,21 @@ template <> struct Fast<float> {
     static __device__ __forceinline__ float rcp(float x) { return frcp_approx(x); }
     static __device__ __forceinline__ float div(float a, float b) { return a * frcp_approx(b); }
 };
+// FP64 vector instructions are what an FP64 update waits for (2 lanes a clock
+// and SM; the divide took most of 98 of them a cell), so 1/x is one
+// third-order Newton (Chebyshev) step from the hardware's 20-bit estimate:
+// with e = 1 - x y, y (1 + e + e^2) = (1 - e^3) / x, three fused operations,
+// within 1 ulp.  x must be normal; an estimate that underflows gives 0, an
+// infinite x NaN.
+__device__ __forceinline__ double drcp_approx(double x)
+{
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = __fma_rn(-x, y, 1.0);
+    return __fma_rn(y, __fma_rn(e, e, e), y);
+}
 template <> struct Fast<double> {
-    static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
+    static __device__ __forceinline__ double rcp(double x) { return drcp_approx(x); }
     static __device__ __forceinline__ double div(double a, double b) { return a / b; }
 };
 
@@ -105,24 +118,126 @@ template <typename R, bool VL> __device__ __forceinline__ R level(int lim, R a, 
 }
 template <> __device__ __forceinline__ float level<float, true>(int, float a, float b) { return vl_level(a, b); }
 
-// PCR over a team of P <= 32 lanes (width-P shuffles), as pcr_warp.
+// The two levels of the nested limiter as one per cell (inner) and one per
+// face (outer); outer's result times Outer::SCALE is L(L(a,b), L(c,d)).
+// FP64 van Leer: L is the harmonic mean, so the nest is
+// 4 / (1/a + 1/b + 1/c + 1/d) where all four share a sign.  A cell keeps
+// w = 1/a + 1/b = (a + b) / (a b) (0 where the signs differ), a face takes
+// 1 / (w_p + w_{p+1}): two reciprocals a cell where the nest of quotients
+// takes two divisions, with the same range (a b must not overflow).  Signs and
+// zeros are told from the high words, off the FP64 pipe; products below the
+// smallest normal number (differences under 1e-154) and non-finite ones give 0.
+template <typename R, bool VL> struct Limit {
+    static constexpr int SCALE = 1;
+    static __device__ __forceinline__ R inner(int lim, R a, R b) { return level<R, VL>(lim, a, b); }
+    static __device__ __forceinline__ R outer(int lim, R v, R w) { return level<R, VL>(lim, v, w); }
+};
+template <> struct Limit<double, true> {
+    static constexpr int SCALE = 4;
+    static __device__ __forceinline__ double inner(int, double a, double b)
+    {
+        const double p = a * b, w = (a + b) * drcp_approx(p);
+        return (unsigned)(__double2hiint(p) - 0x00100000) < 0x7fe00000u ? w : 0.0;
+    }
+    static __device__ __forceinline__ double outer(int, double v, double w)
+    {
+        const int hv = __double2hiint(v), hw = __double2hiint(w);
+        const double r = drcp_approx(v + w);
+        return hv != 0 && hw != 0 && (hv ^ hw) >= 0 ? r : 0.0;
+    }
+};
+
+// NaN or infinity (the exponent bits, off the FP64 pipe).
+__device__ __forceinline__ bool non_finite(float v) { return !(fabsf(v) < INFINITY); }
+__device__ __forceinline__ bool non_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+
+// PCR over a team of P <= 32 lanes (width-P shuffles), as pcr_warp.  Each lane
+// takes the reciprocal of its own diagonal once and hands that on, instead of
+// dividing by both neighbours' diagonals.
 template <typename R> __device__ __forceinline__ R pcr_team(Reduced<R> q, int t, int P)
 {
     const unsigned full = 0xffffffffu;
     for (int h = 1; h < P; h <<= 1) {
         const int tm = (t - h) & (P - 1), tp = (t + h) & (P - 1);
-        const R Lm = __shfl_sync(full, q.L, tm, P), Dm = __shfl_sync(full, q.D, tm, P);
+        const R iD = Fast<R>::rcp(q.D);
+        const R Lm = __shfl_sync(full, q.L, tm, P), iDm = __shfl_sync(full, iD, tm, P);
         const R Um = __shfl_sync(full, q.U, tm, P), Rm = __shfl_sync(full, q.Rr, tm, P);
-        const R Lp = __shfl_sync(full, q.L, tp, P), Dp = __shfl_sync(full, q.D, tp, P);
+        const R Lp = __shfl_sync(full, q.L, tp, P), iDp = __shfl_sync(full, iD, tp, P);
         const R Up = __shfl_sync(full, q.U, tp, P), Rp = __shfl_sync(full, q.Rr, tp, P);
-        const R k1 = Fast<R>::div(q.L, Dm), k2 = Fast<R>::div(q.U, Dp);
+        const R k1 = q.L * iDm, k2 = q.U * iDp;
         q.D = q.D - k1 * Um - k2 * Lp;
         q.Rr = q.Rr - k1 * Rm - k2 * Rp;
         q.L = -k1 * Lm;
         q.U = -k2 * Up;
     }
-    return Fast<R>::div(q.Rr, q.L + q.D + q.U);
+    return q.Rr * Fast<R>::rcp(q.L + q.D + q.U);
 }
+
+// Bottom-up elimination of a segment's rows s .. e-1 into maps delta_k = rho -
+// alp delta_{k-1} - gam X (X = delta_e) and their composite delta_{e-1} = qp +
+// qq delta_{s-1} + qw X, which row e needs.
+template <typename R> struct Segment {
+    R rho = R(0), alp = R(0), gam = R(-1);  // map of the row below: first the virtual row e
+    R qp = R(0), qq = R(1), qw = R(0);
+    // row k: -lgkm d_{k-1} + (1 + lgkm + lgk) d_k - lgk d_{k+1} = Fk - Fkm
+    __device__ __forceinline__ void elim(R Fk, R Fkm, R lgk, R lgkm, R &ro, R &ao, R &go)
+    {
+        const R inv = Fast<R>::rcp((R(1) + lgkm + lgk) + lgk * alp);
+        const R al = -lgkm * inv, ga = lgk * gam * inv, rh = ((Fk - Fkm) + lgk * rho) * inv;
+        ro = rh;
+        ao = al;
+        go = ga;
+        qp = qp + qq * rh;
+        qw = qw - qq * ga;
+        qq = -qq * al;
+        rho = rh;
+        alp = al;
+        gam = ga;
+    }
+    // The equation of X in X_{t-1}, X, X_{t+1}: row e (-lgem, 1 + lgem + lge,
+    // -lge; right-hand side re) with delta_{e-1} and the next segment's first
+    // row (rho_n, alp_n, gam_n) substituted.
+    __device__ __forceinline__ Reduced<R> reduced(R lgem, R lge, R re, R, R rho_n, R alp_n, R gam_n) const
+    {
+        return make_reduced<R>(-lgem, R(1) + lgem + lge, -lge, re, qp, qq, qw, rho_n, alp_n, gam_n);
+    }
+};
+// FP64 carries less: the line matrix is symmetric (-lg_k on both sides of the
+// diagonal), so the product of the alphas is that of the gammas times
+// lg_k / lg_{e-1}, and row e sees the composite only times lg_{e-1}.  With
+// w_k = lg_k gam_{k+1} (a factor of gam_k in any case), lg_{e-1} qp is the sum
+// of -w_k rho_k, lg_{e-1} qw that of w_k gam_k, and lg_{e-1} qq is -gam_s
+// lg_{s-1}: 14 FP64 operations a row, the reciprocal among them, instead of
+// 23 with a division, and no quotient by an lg that may be 0.
+template <> struct Segment<double> {
+    double rho = 0.0, alp = 0.0, gam = -1.0;
+    double A = 0.0, B = 0.0;  // lg_{e-1} qp, lg_{e-1} qw
+    __device__ __forceinline__ void elim(double Fk, double Fkm, double lgk, double lgkm, double &ro, double &ao,
+                                         double &go)
+    {
+        const double inv = Fast<double>::rcp((1.0 + lgkm + lgk) + lgk * alp);
+        const double w = lgk * gam;
+        rho = ((Fk - Fkm) + lgk * rho) * inv;
+        alp = -lgkm * inv;
+        gam = w * inv;
+        A -= w * rho;
+        B += w * gam;
+        ro = rho;
+        ao = alp;
+        go = gam;
+    }
+    // lgs = lg_{s-1}, the face below the segment
+    __device__ __forceinline__ Reduced<double> reduced(double lgem, double lge, double re, double lgs, double rho_n,
+                                                       double alp_n, double gam_n) const
+    {
+        Reduced<double> q;
+        q.L = gam * lgs;
+        q.D = (1.0 + lgem + lge) - B + lge * alp_n;
+        q.U = lge * gam_n;
+        q.Rr = re + A + lge * rho_n;
+        return q;
+    }
+};
 
 // Register budgets.  The FP32 2-D form asks for four resident 256-thread
 // blocks' worth of registers per SM (at most 64 per thread, no spills): lines
@@ -243,7 +358,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
     const C *G = static_cast<const C *>(J.g) + (size_t)lc * n;
     const C *E = static_cast<const C *>(J.e) + (size_t)lc * n;
     const C *E2 = D3 ? static_cast<const C *>(J.e2) + (size_t)lc * n : E;
-    const R lam = (R)J.lam, mu = (R)J.mu, mu2 = (R)J.mu2;
+    typedef Limit<R, VL> LM;
+    const R lam = (R)J.lam, mu = R(LM::SCALE) * (R)J.mu, mu2 = R(LM::SCALE) * (R)J.mu2;
     const R chi_a = (R)J.chi_alpha, chi_it = (R)J.chi_itref;
     auto chi_of = [chi_a, chi_it](R T_) { return T_ > R(0) ? chi_pow<R>(T_ * chi_it, chi_a) : R(0); };
     const unsigned full = 0xffffffffu;
@@ -375,11 +491,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
             R vv[N], ww[N];
             if constexpr (!IMPL) {
 #pragma unroll
-                for (int j = 0; j < N; ++j) vv[j] = level<R, VL>(lim, Tu[j] - Tc[j], Tc[j] - Td[j]);
+                for (int j = 0; j < N; ++j) vv[j] = LM::inner(lim, Tu[j] - Tc[j], Tc[j] - Td[j]);
             }
             if constexpr (D3 && !IMPL) {
 #pragma unroll
-                for (int j = 0; j < N; ++j) ww[j] = level<R, VL>(lim, Tbu[j] - Tc[j], Tc[j] - Tbd[j]);
+                for (int j = 0; j < N; ++j) ww[j] = LM::inner(lim, Tbu[j] - Tc[j], Tc[j] - Tbd[j]);
             }
             R nT = __shfl_down_sync(full, Tc[0], 1, P), nv = R(0), nw = R(0);
             if constexpr (!IMPL) nv = __shfl_down_sync(full, vv[0], 1, P);
@@ -392,11 +508,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
             if (cur == m - 1) {  // the cell after the line
                 if constexpr (!EARLY) {
                     nT = rc[p1];
-                    if constexpr (!IMPL) nv = level<R, VL>(lim, ru[p1] - nT, nT - rd[p1]);
-                    if constexpr (D3 && !IMPL) nw = level<R, VL>(lim, rbu[p1] - nT, nT - rbd[p1]);
+                    if constexpr (!IMPL) nv = LM::inner(lim, ru[p1] - nT, nT - rd[p1]);
+                    if constexpr (D3 && !IMPL) nw = LM::inner(lim, rbu[p1] - nT, nT - rbd[p1]);
                 } else {
                     nT = eT;
-                    if constexpr (!IMPL) nv = level<R, VL>(lim, eU - nT, nT - eD);
+                    if constexpr (!IMPL) nv = LM::inner(lim, eU - nT, nT - eD);
                 }
             }
             Tcar = __shfl_sync(full, Tc[0], 0, P);
@@ -421,11 +537,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
                 } else {
                     const R vnx = j + 1 < N ? vv[j + 1] : nv;
                     const R ej = NL ? Ev[j] * hf[j] : Ev[j];
-                    F[j] = lg[j] * (Tnx - Tc[j]) + mu * ej * level<R, VL>(lim, vv[j], vnx);
+                    F[j] = lg[j] * (Tnx - Tc[j]) + mu * ej * LM::outer(lim, vv[j], vnx);
                 }
                 if constexpr (D3 && !IMPL) {
                     const R wnx = j + 1 < N ? ww[j + 1] : nw;
-                    F[j] += mu2 * (NL ? E2v[j] * hf[j] : E2v[j]) * level<R, VL>(lim, ww[j], wnx);
+                    F[j] += mu2 * (NL ? E2v[j] * hf[j] : E2v[j]) * LM::outer(lim, ww[j], wnx);
                 }
             }
             if (c < m) {
@@ -437,25 +553,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
     __syncwarp();
 
     // ---- B1: bottom-up elimination of lane t's segment
-    R rho1 = R(0), alp1 = R(0), gam1 = R(-1);
-    R qp = R(0), qq = R(1), qw = R(0);
-    R ae = R(0), be = R(1), ce = R(0), re = R(0);
+    Segment<R> sg;
+    R lgem = R(0), lge = R(0), re = R(0), lgs = R(0);
     {
-        auto elim = [&](R Fk, R Fkm, R lgk, R lgkm, R &ro_, R &ao_, R &go_) {
-            // row k: -lgkm d_{k-1} + (1 + lgkm + lgk) d_k - lgk d_{k+1} = Fk - Fkm
-            const R inv = Fast<R>::rcp((R(1) + lgkm + lgk) + lgk * alp1);
-            const R alp = -lgkm * inv, gam = lgk * gam1 * inv, rho = ((Fk - Fkm) + lgk * rho1) * inv;
-            ro_ = rho;
-            ao_ = alp;
-            go_ = gam;
-            qp = qp + qq * rho;
-            qw = qw - qq * gam;
-            qq = -qq * alp;
-            rho1 = rho;
-            alp1 = alp;
-            gam1 = gam;
-        };
-        R Fpend = R(0), lgpend = R(0), Flast = R(0), lglast = R(0);
+        R Fpend = R(0), lgpend = R(0), Flast = R(0);
         R ro[N], ao[N], go[N];  // maps of the chunk above, waiting for its row 0
 #pragma unroll
         for (int v = 0; v < N; ++v) ro[v] = ao[v] = go[v] = R(0);
@@ -473,18 +574,16 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
             V16<R>::unpack(sB[swz(c)], lg);
             if (u == Ut - 1) {
                 // row e (last cell of the segment) enters the reduced system
-                ae = -lg[N - 2];
-                ce = -lg[N - 1];
-                be = R(1) - ae - ce;
+                lge = lg[N - 1];
+                lgem = lg[N - 2];
                 re = F[N - 1] - F[N - 2];
                 Flast = F[N - 1];
-                lglast = lg[N - 1];
                 co[N - 1] = cao[N - 1] = cgo[N - 1] = R(0);
 #pragma unroll
-                for (int j = N - 2; j >= 1; --j) elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
+                for (int j = N - 2; j >= 1; --j) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             } else {
                 // row 0 of the chunk above, then this chunk's rows N-1 .. 1
-                elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
+                sg.elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
                 sA[swz(c + 1)] = V16<R>::pack(ro);
                 sB[swz(c + 1)] = V16<R>::pack(ao);
                 if constexpr (TM) {
@@ -494,7 +593,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
                     sC[swz(c + 1)] = V16<R>::pack(go);
                 }
 #pragma unroll
-                for (int j = N - 1; j >= 1; --j) elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
+                for (int j = N - 1; j >= 1; --j) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             }
             Fpend = F[0];
             lgpend = lg[0];
@@ -511,8 +610,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
         }
         // row s needs the face below the segment: the previous lane's last face
         const int tp = (t - 1) & (P - 1);
-        const R Fprev = __shfl_sync(full, Flast, tp, P), lgprev = __shfl_sync(full, lglast, tp, P);
-        elim(Fpend, Fprev, lgpend, lgprev, ro[0], ao[0], go[0]);
+        const R Fprev = __shfl_sync(full, Flast, tp, P), lgprev = __shfl_sync(full, lge, tp, P);
+        lgs = lgprev;
+        sg.elim(Fpend, Fprev, lgpend, lgprev, ro[0], ao[0], go[0]);
         sA[swz(c_lo)] = V16<R>::pack(ro);
         sB[swz(c_lo)] = V16<R>::pack(ao);
         if constexpr (TM) {
@@ -537,9 +637,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
     R X, Xm;
     {
         const int tn = (t + 1) & (P - 1);
-        const R rho_n = __shfl_sync(full, rho1, tn, P), alp_n = __shfl_sync(full, alp1, tn, P),
-                gam_n = __shfl_sync(full, gam1, tn, P);
-        X = pcr_team<R>(make_reduced<R>(ae, be, ce, re, qp, qq, qw, rho_n, alp_n, gam_n), t, P);
+        const R rho_n = __shfl_sync(full, sg.rho, tn, P), alp_n = __shfl_sync(full, sg.alp, tn, P),
+                gam_n = __shfl_sync(full, sg.gam, tn, P);
+        X = pcr_team<R>(sg.reduced(lgem, lge, re, lgs, rho_n, alp_n, gam_n), t, P);
         Xm = __shfl_sync(full, X, (t - 1) & (P - 1), P);
     }
 
@@ -589,10 +689,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 to[j] += d[j];
-                sum += to[j];
+                if constexpr (N == 4) sum += to[j];  // FP32: one test for the chunk
+                else bad |= non_finite(to[j]);
             }
-            bad |= !(fabs(sum) < R(INFINITY));  // a NaN or infinity in the chunk
+            if constexpr (N == 4) bad |= non_finite(sum);
             if (diag && active) {
+                if constexpr (N != 4) sum = to[0] + to[1];
                 const R y = sum - dl, tt = dh + y;
                 dl = (tt - dh) - y;
                 dh = tt;

@@ -471,13 +471,14 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
         }
         for (int h = 1; h < 32; h <<= 1) {
             const int tm = (lane - h) & 31, tp = (lane + h) & 31;
-            const R Lm = __shfl_sync(full, q.L, tm), Dm = __shfl_sync(full, q.D, tm);
+            const R iD = Fast<R>::rcp(q.D);
+            const R Lm = __shfl_sync(full, q.L, tm), iDm = __shfl_sync(full, iD, tm);
             const R Um = __shfl_sync(full, q.U, tm), Rm = __shfl_sync(full, q.Rr, tm);
             const R Qm = __shfl_sync(full, Q, tm), Wm = __shfl_sync(full, W, tm);
-            const R Lp = __shfl_sync(full, q.L, tp), Dp = __shfl_sync(full, q.D, tp);
+            const R Lp = __shfl_sync(full, q.L, tp), iDp = __shfl_sync(full, iD, tp);
             const R Up = __shfl_sync(full, q.U, tp), Rp = __shfl_sync(full, q.Rr, tp);
             const R Qp = __shfl_sync(full, Q, tp), Wp = __shfl_sync(full, W, tp);
-            const R k1 = Fast<R>::div(q.L, Dm), k2 = Fast<R>::div(q.U, Dp);
+            const R k1 = q.L * iDm, k2 = q.U * iDp;
             q.D = q.D - k1 * Um - k2 * Lp;
             q.Rr = q.Rr - k1 * Rm - k2 * Rp;
             Q = Q - k1 * Qm - k2 * Qp;
