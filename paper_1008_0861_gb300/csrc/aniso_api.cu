@@ -427,7 +427,7 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
         CU(cudaEventRecordWithFlags(h->prof.pool[pidx].a, s, rec_flags));
     }
     CU(v7   ? launch_line7(h->field_fp16, a, cs, smem, s)
-       : v6 ? launch_line6(h->field_fp16, a, J.nblocks, nthreads, smem, s)
+       : v6 ? launch_line6(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s)
        : v4 ? launch_line4(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s)
             : launch_line2(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s, in_lo != nullptr));
     if (h->profile) {
@@ -1572,7 +1572,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             a.limiter = b->hs[0]->limiter;
             a.err = err;
             a.block_job = reinterpret_cast<const int *>(static_cast<unsigned char *>(b->d_jobs) + L.table);
-            return launch_line6(fp16, a, L.nblocks, L.nthreads, L.smem, st);
+            return launch_line6(prec, fp16, a, L.nblocks, L.nthreads, L.smem, st);
         }
         if (L.kind == 9 || L.kind == 10) {
             Line5Args a{};

@@ -140,6 +140,8 @@ cudaError_t launch_diag_finish(const Line2Job *jobs, int njobs, const DiagPart *
 // ring[0 .. count) = NaN (slots no step writes read as NaN).
 cudaError_t launch_fill_nan(double *ring, size_t count, cudaStream_t s);
 constexpr int MAX_LINE2_TRANSPOSED = 2048;
+// Longest FP64 line of the warp-per-line kernel with its default segments (16 chunks of 2 cells on 32 lanes).
+constexpr int MAX_LINE4_FP64 = 1024;
 
 // Launch configuration helpers (host).
 // line2: returns false when the line cannot use the vectorised kernel.
@@ -174,11 +176,13 @@ bool line4_config(int prec, int n, bool transposed, int warps, int seg_chunks, i
                   int *nthreads, size_t *smem, bool tmem = false);
 cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads,
                          size_t smem, cudaStream_t s);
-// Long lines (line6): 2048 < n <= 4096, FP32, teams of 128 lanes over four
-// warps, `lines` (4 or 2) lines per block.  False when the line does not fit.
+// Long lines (line6): FP32 2048 < n <= 4096, FP64 1024 < n <= 4096, teams of
+// 128 lanes over four warps; FP32 `lines` (4 or 2) lines per block, FP64 two.
+// False when the line does not fit.
 bool line6_config(int prec, int coef_fp16, int n, int *team, int *lines_per_block, int *nthreads, size_t *smem,
                   int lines = 4);
-cudaError_t launch_line6(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s);
+cudaError_t launch_line6(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
+                         cudaStream_t s);
 // Lines cut across a thread-block cluster (line7): FP32, n = cs * np with
 // np = 2048 (else 1024) and cs = 1, 2, 4 or 8; four lines a block, one job
 // (args.one) a launch; with TinLo/ToutLo set, the compensated state; with

@@ -79,11 +79,11 @@ template <> struct Fast<float> {
     static __device__ __forceinline__ float div(float a, float b) { return a * frcp_approx(b); }
 };
 // FP64 vector instructions are what an FP64 update waits for (2 lanes a clock
-// and SM; the divide took most of 98 of them a cell), so 1/x is one
-// third-order Newton (Chebyshev) step from the hardware's 20-bit estimate:
-// with e = 1 - x y, y (1 + e + e^2) = (1 - e^3) / x, three fused operations,
-// within 1 ulp.  x must be normal; an estimate that underflows gives 0, an
-// infinite x NaN.
+// and SM), and divisions were most of its 98 a cell.  1/x here is one
+// third-order Newton step (Chebyshev's method) from the hardware's 20-bit
+// estimate: with e = 1 - x y, y (1 + e + e^2) = (1 - e^3) / x, three fused
+// operations, within 1 ulp.  x must be normal; an estimate that underflows
+// gives 0, an infinite x NaN.
 __device__ __forceinline__ double drcp_approx(double x)
 {
     double y;
@@ -91,8 +91,21 @@ __device__ __forceinline__ double drcp_approx(double x)
     const double e = __fma_rn(-x, y, 1.0);
     return __fma_rn(y, __fma_rn(e, e, e), y);
 }
+// Correctly rounded quotient and reciprocal from such a y: one step with the
+// exact remainder (Markstein, IBM J. Res. Dev. 34, 1990), the same bits as an
+// IEEE division wherever remainder and quotient are normal numbers.
+__device__ __forceinline__ double dquot(double a, double b, double y)
+{
+    const double q = a * y;
+    return __fma_rn(__fma_rn(-b, q, a), y, q);
+}
+__device__ __forceinline__ double drcp(double x)
+{
+    const double y = drcp_approx(x);
+    return __fma_rn(__fma_rn(-x, y, 1.0), y, y);
+}
 template <> struct Fast<double> {
-    static __device__ __forceinline__ double rcp(double x) { return drcp_approx(x); }
+    static __device__ __forceinline__ double rcp(double x) { return drcp(x); }
     static __device__ __forceinline__ double div(double a, double b) { return a / b; }
 };
 
@@ -119,20 +132,35 @@ template <typename R, bool VL> __device__ __forceinline__ R level(int lim, R a, 
 template <> __device__ __forceinline__ float level<float, true>(int, float a, float b) { return vl_level(a, b); }
 
 // The two levels of the nested limiter as one per cell (inner) and one per
-// face (outer); outer's result times Outer::SCALE is L(L(a,b), L(c,d)).
-// FP64 van Leer: L is the harmonic mean, so the nest is
-// 4 / (1/a + 1/b + 1/c + 1/d) where all four share a sign.  A cell keeps
-// w = 1/a + 1/b = (a + b) / (a b) (0 where the signs differ), a face takes
-// 1 / (w_p + w_{p+1}): two reciprocals a cell where the nest of quotients
-// takes two divisions, with the same range (a b must not overflow).  Signs and
-// zeros are told from the high words, off the FP64 pipe; products below the
-// smallest normal number (differences under 1e-154) and non-finite ones give 0.
-template <typename R, bool VL> struct Limit {
+// face (outer); outer's result times SCALE is L(L(a,b), L(c,d)).
+template <typename R, bool VL, bool HARMONIC = false> struct Limit {
     static constexpr int SCALE = 1;
     static __device__ __forceinline__ R inner(int lim, R a, R b) { return level<R, VL>(lim, a, b); }
     static __device__ __forceinline__ R outer(int lim, R v, R w) { return level<R, VL>(lim, v, w); }
 };
-template <> struct Limit<double, true> {
+// FP64 van Leer, the nest as written: a cell keeps ab / (a + b), half of its
+// level, a face forms the same quotient of two cells', a quarter of the nest
+// (powers of two: the bits of the nest of 2ab / (a + b)).  Signs and zeros are
+// told from the high words, off the FP64 pipe; products below the smallest
+// normal number (differences under 1e-154) and non-finite ones give 0.
+// A run amplifies the last bit (the ring at 1000 times the limit by 1e6 in a
+// hundred steps), which is why the quotients keep their rounding.
+template <> struct Limit<double, true, false> {
+    static constexpr int SCALE = 4;
+    static __device__ __forceinline__ double inner(int, double a, double b)
+    {
+        const double p = a * b, s = a + b;
+        const double q = dquot(p, s, drcp_approx(s));
+        return (unsigned)(__double2hiint(p) - 0x00100000) < 0x7fe00000u ? q : 0.0;
+    }
+    static __device__ __forceinline__ double outer(int lim, double v, double w) { return inner(lim, v, w); }
+};
+// FP64 van Leer by sums of reciprocals (the long lines, whose segments are
+// others than they were): L is the harmonic mean, so the nest is
+// 4 / (1/a + 1/b + 1/c + 1/d) where all four share a sign.  A cell keeps
+// w = 1/a + 1/b = (a + b) / (a b) (0 where the signs differ), a face takes
+// 1 / (w_p + w_{p+1}): 12 operations a cell instead of 18, the same range.
+template <> struct Limit<double, true, true> {
     static constexpr int SCALE = 4;
     static __device__ __forceinline__ double inner(int, double a, double b)
     {
@@ -153,30 +181,40 @@ __device__ __forceinline__ bool non_finite(double v) { return (__double2hiint(v)
 
 // PCR over a team of P <= 32 lanes (width-P shuffles), as pcr_warp.  Each lane
 // takes the reciprocal of its own diagonal once and hands that on, instead of
-// dividing by both neighbours' diagonals.
+// dividing by both neighbours' diagonals (the quotients' bits are kept).
+__device__ __forceinline__ float pcr_ratio(float a, float, float y) { return a * y; }
+__device__ __forceinline__ double pcr_ratio(double a, double b, double y) { return dquot(a, b, y); }
+__device__ __forceinline__ float pcr_recip(float x) { return frcp_approx(x); }
+__device__ __forceinline__ double pcr_recip(double x) { return drcp_approx(x); }
 template <typename R> __device__ __forceinline__ R pcr_team(Reduced<R> q, int t, int P)
 {
     const unsigned full = 0xffffffffu;
     for (int h = 1; h < P; h <<= 1) {
         const int tm = (t - h) & (P - 1), tp = (t + h) & (P - 1);
-        const R iD = Fast<R>::rcp(q.D);
+        const R iD = pcr_recip(q.D);
+        R Dm = R(0), Dp = R(0);
+        if constexpr (sizeof(R) == 8) {  // the remainders' divisors
+            Dm = __shfl_sync(full, q.D, tm, P);
+            Dp = __shfl_sync(full, q.D, tp, P);
+        }
         const R Lm = __shfl_sync(full, q.L, tm, P), iDm = __shfl_sync(full, iD, tm, P);
         const R Um = __shfl_sync(full, q.U, tm, P), Rm = __shfl_sync(full, q.Rr, tm, P);
         const R Lp = __shfl_sync(full, q.L, tp, P), iDp = __shfl_sync(full, iD, tp, P);
         const R Up = __shfl_sync(full, q.U, tp, P), Rp = __shfl_sync(full, q.Rr, tp, P);
-        const R k1 = q.L * iDm, k2 = q.U * iDp;
+        const R k1 = pcr_ratio(q.L, Dm, iDm), k2 = pcr_ratio(q.U, Dp, iDp);
         q.D = q.D - k1 * Um - k2 * Lp;
         q.Rr = q.Rr - k1 * Rm - k2 * Rp;
         q.L = -k1 * Lm;
         q.U = -k2 * Up;
     }
-    return q.Rr * Fast<R>::rcp(q.L + q.D + q.U);
+    const R D = q.L + q.D + q.U;
+    return pcr_ratio(q.Rr, D, pcr_recip(D));
 }
 
 // Bottom-up elimination of a segment's rows s .. e-1 into maps delta_k = rho -
 // alp delta_{k-1} - gam X (X = delta_e) and their composite delta_{e-1} = qp +
 // qq delta_{s-1} + qw X, which row e needs.
-template <typename R> struct Segment {
+template <typename R, bool SYMMETRIC = false> struct Segment {
     R rho = R(0), alp = R(0), gam = R(-1);  // map of the row below: first the virtual row e
     R qp = R(0), qq = R(1), qw = R(0);
     // row k: -lgkm d_{k-1} + (1 + lgkm + lgk) d_k - lgk d_{k+1} = Fk - Fkm
@@ -202,20 +240,20 @@ template <typename R> struct Segment {
         return make_reduced<R>(-lgem, R(1) + lgem + lge, -lge, re, qp, qq, qw, rho_n, alp_n, gam_n);
     }
 };
-// FP64 carries less: the line matrix is symmetric (-lg_k on both sides of the
-// diagonal), so the product of the alphas is that of the gammas times
-// lg_k / lg_{e-1}, and row e sees the composite only times lg_{e-1}.  With
-// w_k = lg_k gam_{k+1} (a factor of gam_k in any case), lg_{e-1} qp is the sum
-// of -w_k rho_k, lg_{e-1} qw that of w_k gam_k, and lg_{e-1} qq is -gam_s
-// lg_{s-1}: 14 FP64 operations a row, the reciprocal among them, instead of
-// 23 with a division, and no quotient by an lg that may be 0.
-template <> struct Segment<double> {
+// SYMMETRIC (FP64, the long lines) carries less: the line matrix is symmetric
+// (-lg_k on both sides of the diagonal), so the product of the alphas is that
+// of the gammas times lg_k / lg_{e-1}, and row e sees the composite only times
+// lg_{e-1}.  With w_k = lg_k gam_{k+1} (a factor of gam_k in any case),
+// lg_{e-1} qp is the sum of -w_k rho_k, lg_{e-1} qw that of w_k gam_k, and
+// lg_{e-1} qq is -gam_s lg_{s-1}: 14 FP64 operations a row instead of 17, and
+// no quotient by an lg that may be 0.
+template <> struct Segment<double, true> {
     double rho = 0.0, alp = 0.0, gam = -1.0;
     double A = 0.0, B = 0.0;  // lg_{e-1} qp, lg_{e-1} qw
     __device__ __forceinline__ void elim(double Fk, double Fkm, double lgk, double lgkm, double &ro, double &ao,
                                          double &go)
     {
-        const double inv = Fast<double>::rcp((1.0 + lgkm + lgk) + lgk * alp);
+        const double inv = drcp_approx((1.0 + lgkm + lgk) + lgk * alp);
         const double w = lgk * gam;
         rho = ((Fk - Fkm) + lgk * rho) * inv;
         alp = -lgkm * inv;

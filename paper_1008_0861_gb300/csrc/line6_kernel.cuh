@@ -1,7 +1,8 @@
-// line6_kernel.cuh -- long lines (2048 < n <= 4096 cells, FP32): the
-// warp-autonomous line kernel's phases with a line's team spread over W
-// warps (P = 32 W lanes), so that a block still holds four lines and the
-// transposed store still writes 16-byte pieces.
+// line6_kernel.cuh -- long lines (FP32: 2048 < n <= 4096 cells; FP64: 1024 < n
+// <= 4096): the warp-autonomous line kernel's phases with a line's team spread
+// over W warps (P = 32 W lanes), so that a block still holds a vector's worth
+// of lines (four in FP32, two in FP64) and the transposed store still writes
+// 16-byte pieces.
 //
 // Same linear algebra and the same per-lane work as line4 (delta form,
 // coalesced flux phase, bottom-up segment elimination in shared memory,
@@ -24,12 +25,40 @@
 
 namespace aniso {
 
-template <typename C, bool VL>
+// PCR through shared memory as pcr_smem, each thread handing on the reciprocal
+// of its diagonal (FP64: one reciprocal a level instead of two divisions).
+__device__ __forceinline__ double pcr_team_smem(Reduced<double> q, int t, int P, double *sL, double *sI, double *sU,
+                                                double *sR)
+{
+    for (int h = 1; h < P; h <<= 1) {
+        sL[t] = q.L;
+        sI[t] = drcp_approx(q.D);
+        sU[t] = q.U;
+        sR[t] = q.Rr;
+        __syncthreads();
+        const int tm = (t - h) & (P - 1), tp = (t + h) & (P - 1);
+        const double k1 = q.L * sI[tm], k2 = q.U * sI[tp];
+        q.D = q.D - k1 * sU[tm] - k2 * sL[tp];
+        q.Rr = q.Rr - k1 * sR[tm] - k2 * sR[tp];
+        q.L = -k1 * sL[tm];
+        q.U = -k2 * sU[tp];
+        __syncthreads();
+    }
+    return q.Rr * drcp_approx(q.L + q.D + q.U);
+}
+__device__ __forceinline__ float pcr_team_smem(Reduced<float> q, int t, int P, float *sL, float *sD, float *sU,
+                                               float *sR)
+{
+    return pcr_smem<float>(q, t, P, sL, sD, sU, sR, 1);
+}
+
+template <typename R, typename C, bool VL>
 __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
 {
-    typedef float R;
-    typedef float4 VT;
-    constexpr int N = 4;
+    typedef typename V16<R>::T VT;
+    typedef Limit<R, VL, true> LM;
+    constexpr int N = V16<R>::N;
+    constexpr int LOGN = N == 4 ? 2 : 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Line2Job J;
     if (args.jobs) {  // the block's job, copied by warp 0's lanes a word each
@@ -62,7 +91,7 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
     const R *rc = Tin + (size_t)lc * n, *ru = Tin + (size_t)lu * n, *rd = Tin + (size_t)ld * n;
     const C *G = static_cast<const C *>(J.g) + (size_t)lc * n;
     const C *E = static_cast<const C *>(J.e) + (size_t)lc * n;
-    const R lam = (R)J.lam, mu = (R)J.mu;
+    const R lam = (R)J.lam, mu = R(LM::SCALE) * (R)J.mu;
     const unsigned full = 0xffffffffu;
 
     if (threadIdx.x == 0) {  // the block's rows into L2 (a hint)
@@ -132,11 +161,11 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
             unpack_raw(x.e, Ev);
             R vv[N];
 #pragma unroll
-            for (int j = 0; j < N; ++j) vv[j] = level<R, VL>(lim, Tu[j] - Tc[j], Tc[j] - Td[j]);
+            for (int j = 0; j < N; ++j) vv[j] = LM::inner(lim, Tu[j] - Tc[j], Tc[j] - Td[j]);
             R nT = __shfl_down_sync(full, Tc[0], 1), nv = __shfl_down_sync(full, vv[0], 1);
             if (lane == 31 || x.cur == m - 1) {
                 nT = x.nc;
-                nv = level<R, VL>(lim, x.nu - nT, nT - x.nd);
+                nv = LM::inner(lim, x.nu - nT, nT - x.nd);
             }
             R F[N], lg[N];
 #pragma unroll
@@ -144,7 +173,7 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
                 const R Tnx = j + 1 < N ? Tc[j + 1] : nT;
                 const R vnx = j + 1 < N ? vv[j + 1] : nv;
                 lg[j] = lam * Gv[j];
-                F[j] = lg[j] * (Tnx - Tc[j]) + mu * Ev[j] * level<R, VL>(lim, vv[j], vnx);
+                F[j] = lg[j] * (Tnx - Tc[j]) + mu * Ev[j] * LM::outer(lim, vv[j], vnx);
             }
             if (c < m) {
                 sA[swz(c)] = V16<R>::pack(F);
@@ -155,25 +184,10 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
     __syncthreads();
 
     // ---- B1: bottom-up elimination of lane t's segment
-    R rho1 = R(0), alp1 = R(0), gam1 = R(-1);
-    R qp = R(0), qq = R(1), qw = R(0);
-    R ae = R(0), be = R(1), ce = R(0), re = R(0);
-    R Fpend = R(0), lgpend = R(0), Flast = R(0), lglast = R(0);
+    Segment<R, sizeof(R) == 8> sg;
+    R lgem = R(0), lge = R(0), re = R(0), lgs;
+    R Fpend = R(0), lgpend = R(0), Flast = R(0);
     R ro[N], ao[N], go[N];  // maps of the chunk above, waiting for its row 0
-    auto elim = [&](R Fk, R Fkm, R lgk, R lgkm, R &ro_, R &ao_, R &go_) {
-        // row k: -lgkm d_{k-1} + (1 + lgkm + lgk) d_k - lgk d_{k+1} = Fk - Fkm
-        const R inv = Fast<R>::rcp((R(1) + lgkm + lgk) + lgk * alp1);
-        const R alp = -lgkm * inv, gam = lgk * gam1 * inv, rho = ((Fk - Fkm) + lgk * rho1) * inv;
-        ro_ = rho;
-        ao_ = alp;
-        go_ = gam;
-        qp = qp + qq * rho;
-        qw = qw - qq * gam;
-        qq = -qq * alp;
-        rho1 = rho;
-        alp1 = alp;
-        gam1 = gam;
-    };
     {
 #pragma unroll
         for (int v = 0; v < N; ++v) ro[v] = ao[v] = go[v] = R(0);
@@ -184,23 +198,21 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
             V16<R>::unpack(sB[swz(c)], lg);
             if (u == Ut - 1) {
                 // row e (last cell of the segment) enters the reduced system
-                ae = -lg[N - 2];
-                ce = -lg[N - 1];
-                be = R(1) - ae - ce;
+                lgem = lg[N - 2];
+                lge = lg[N - 1];
                 re = F[N - 1] - F[N - 2];
                 Flast = F[N - 1];
-                lglast = lg[N - 1];
                 co[N - 1] = cao[N - 1] = cgo[N - 1] = R(0);
 #pragma unroll
-                for (int j = N - 2; j >= 1; --j) elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
+                for (int j = N - 2; j >= 1; --j) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             } else {
                 // row 0 of the chunk above, then this chunk's rows N-1 .. 1
-                elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
+                sg.elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
                 sA[swz(c + 1)] = V16<R>::pack(ro);
                 sB[swz(c + 1)] = V16<R>::pack(ao);
                 sC[swz(c + 1)] = V16<R>::pack(go);
 #pragma unroll
-                for (int j = N - 1; j >= 1; --j) elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
+                for (int j = N - 1; j >= 1; --j) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             }
             Fpend = F[0];
             lgpend = lg[0];
@@ -214,11 +226,12 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
     }
     // row s needs the face below the segment: the previous lane's last face
     ex0[t] = Flast;
-    ex1[t] = lglast;
+    ex1[t] = lge;
     __syncthreads();
     {
         const int tp = (t - 1 + P) % P;
-        elim(Fpend, ex0[tp], lgpend, ex1[tp], ro[0], ao[0], go[0]);
+        lgs = ex1[tp];
+        sg.elim(Fpend, ex0[tp], lgpend, lgs, ro[0], ao[0], go[0]);
         sA[swz(c_lo)] = V16<R>::pack(ro);
         sB[swz(c_lo)] = V16<R>::pack(ao);
         sC[swz(c_lo)] = V16<R>::pack(go);
@@ -233,15 +246,14 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
     // ---- R: reduced system of the line in the segment-end unknowns
     R X, Xm;
     {
-        ex0[t] = rho1;
-        ex1[t] = alp1;
-        ex2[t] = gam1;
+        ex0[t] = sg.rho;
+        ex1[t] = sg.alp;
+        ex2[t] = sg.gam;
         __syncthreads();
         const int tn = (t + 1) % P;
         const R rho_n = ex0[tn], alp_n = ex1[tn], gam_n = ex2[tn];
         __syncthreads();
-        X = pcr_smem<R>(make_reduced<R>(ae, be, ce, re, qp, qq, qw, rho_n, alp_n, gam_n), t, P, ex0, ex1, ex2,
-                        ex3, 1);
+        X = pcr_team_smem(sg.reduced(lgem, lge, re, lgs, rho_n, alp_n, gam_n), t, P, ex0, ex1, ex2, ex3);
         ex0[t] = X;
         __syncthreads();
         Xm = ex0[(t - 1 + P) % P];
@@ -280,9 +292,10 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             to[j] += d[j];
-            sum += to[j];
+            if constexpr (N == 4) sum += to[j];
+            else bad |= non_finite(to[j]);
         }
-        bad |= !(fabsf(sum) < INFINITY);
+        if constexpr (N == 4) bad |= non_finite(sum);
         if (!J.transpose_out) {
             if (active) reinterpret_cast<VT *>(static_cast<R *>(J.Tout) + (size_t)lc * n)[c] = V16<R>::pack(to);
         } else {
@@ -294,32 +307,34 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
     if (J.transpose_out) {
         __syncthreads();
         R *out = static_cast<R *>(J.Tout);
-        const int groups = LPB >> 2;
-        const bool vec_ok = (nl & 3) == 0;
-        if (LPB == 2) {  // two lines: 8-byte pieces
-            for (int p = threadIdx.x; p < n; p += blockDim.x) {
-                const int sc = swz(p >> 2), j = p & 3;
-                const R o0 = reinterpret_cast<const R *>(reinterpret_cast<const VT *>(smem_raw) + sc)[j];
-                const R o1 = reinterpret_cast<const R *>(reinterpret_cast<const VT *>(smem_raw) + 3 * m + sc)[j];
-                R *dst = out + (size_t)p * nl + line0;
-                if ((nl & 1) == 0 && line0 + 2 <= nl) {
-                    *reinterpret_cast<float2 *>(dst) = make_float2(o0, o1);
-                } else {
-                    if (line0 < nl) dst[0] = o0;
-                    if (line0 + 1 < nl) dst[1] = o1;
+        const int groups = LPB >> LOGN;
+        const bool vec_ok = (nl & (N - 1)) == 0;
+        if constexpr (N == 4) {
+            if (LPB == 2) {  // two lines: 8-byte pieces
+                for (int p = threadIdx.x; p < n; p += blockDim.x) {
+                    const int sc = swz(p >> 2), j = p & 3;
+                    const R o0 = reinterpret_cast<const R *>(reinterpret_cast<const VT *>(smem_raw) + sc)[j];
+                    const R o1 = reinterpret_cast<const R *>(reinterpret_cast<const VT *>(smem_raw) + 3 * m + sc)[j];
+                    R *dst = out + (size_t)p * nl + line0;
+                    if ((nl & 1) == 0 && line0 + 2 <= nl) {
+                        *reinterpret_cast<float2 *>(dst) = make_float2(o0, o1);
+                    } else {
+                        if (line0 < nl) dst[0] = o0;
+                        if (line0 + 1 < nl) dst[1] = o1;
+                    }
                 }
             }
         }
         for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int sc = swz(p >> 2), j = p & 3;
+            const int sc = swz(p >> LOGN), j = p & (N - 1);
             for (int grp = 0; grp < groups; ++grp) {
                 R o[N];
 #pragma unroll
                 for (int i = 0; i < N; ++i) {
-                    const int l = (grp << 2) + i;
+                    const int l = (grp << LOGN) + i;
                     o[i] = reinterpret_cast<const R *>(reinterpret_cast<const VT *>(smem_raw) + (size_t)l * 3 * m + sc)[j];
                 }
-                const int l0 = line0 + (grp << 2);
+                const int l0 = line0 + (grp << LOGN);
                 R *dst = out + (size_t)p * nl + l0;
                 if (vec_ok && l0 + N <= nl) {
                     *reinterpret_cast<VT *>(dst) = V16<R>::pack(o);
