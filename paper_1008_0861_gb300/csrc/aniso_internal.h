@@ -195,6 +195,8 @@ cudaError_t launch_line7(int coef_fp16, const Line2Args &a, int cs, size_t smem,
 // form also capped by the block's TMEM columns, tm_cols), or -1.
 int line4_blocks_per_sm(int prec, int coef_fp16, int limiter, int nthreads, size_t smem, bool tmem = false,
                         int tm_cols = 64);
+// seg_chunks for an FP64 update of nlines lines of n cells launched alone.
+int line4_seg_fp64(int n, int nlines);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.
 int line4_tm_cols(int n, int team);
 // Chunks of padding after each warp's shared area in the FP32 line4 kernel

@@ -76,6 +76,35 @@ int line4_tm_cols(int n, int team)
     return 8 * V <= 32 ? 32 : 64;
 }
 
+// Chunks per lane for one FP64 grid's update on its own.  The FP64 unit of an
+// SM quarter takes a warp instruction every 64 clocks however many lanes it
+// serves, so an update takes as long as the FP64 instructions of the warps
+// that share a quarter: about 43 a cell and 15 a level of the reduced system
+// a lane, 40 besides.  Longer segments give fewer, longer warps; the team with
+// the least for the most loaded of the 4 x 152 quarters wins, from the general
+// rule's team (4 chunks a lane) upwards and that one at equal cost.  50^2:
+// 28.6 us an update with 4 chunks a lane, 11.9 with 1; 128^2: 19.0 and 12.5;
+// from 256 cells a line on both rules agree.
+int line4_seg_fp64(int n, int nlines)
+{
+    const int m = n / 2;
+    int P = 1, top = 1, best = 4;
+    while (P * 2 <= m / 4 && P < 32) P *= 2;
+    while (top * 2 <= m && top < 32) top *= 2;
+    long best_cost = -1;
+    for (; P <= top; P *= 2) {
+        const long warps = ((long)nlines * P + 31) / 32, rounds = (warps + 607) / 608;
+        long levels = 0;
+        while ((1 << levels) < P) ++levels;
+        const long cost = rounds * (2L * 43 * ((m + P - 1) / P) + 15 * levels + 40);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = m / P;  // pow2floor(m / (m / P)) == P
+        }
+    }
+    return best;
+}
+
 // The kernel keeps 16-byte chunk c of a line at c ^ ((c >> s) & 7) inside
 // its group of 8 chunks (the last, incomplete group unswizzled).  The
 // coalesced phases have the 8 lanes of a quarter warp touch one whole group,
