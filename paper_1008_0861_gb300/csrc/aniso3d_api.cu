@@ -157,7 +157,7 @@ extern "C" int aniso3_set_field(aniso3_t h, const void *bx, const void *by, cons
         CU(cudaMalloc(&h->s1, bytes));
         CU(cudaMalloc(&h->s2, bytes));
         CU(cudaMalloc(&h->partials, 4 * TOTALS_BLOCKS * sizeof(double)));
-        CU(cudaMalloc(&h->result, 4 * sizeof(double)));
+        CU(cudaMalloc(&h->result, TOTALS_RESULT * sizeof(double)));
         CU(cudaMalloc(&h->err, sizeof(unsigned)));
         CU(cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->stream));
     }
@@ -240,15 +240,20 @@ extern "C" int aniso3_step(aniso3_t h, void *T, double dt, int nsteps)
     return ANISO_OK;
 }
 
-static int check_err3(aniso3_ctx *h)
+static int report_err3(aniso3_ctx *h, unsigned flag)
 {
-    unsigned flag = 0;
-    CU(cudaMemcpy(&flag, h->err, sizeof flag, cudaMemcpyDeviceToHost));
     if (flag) {
         CU(cudaMemset(h->err, 0, sizeof(unsigned)));
         return fail(ANISO_ERR_NONFINITE, "a 3-D step produced a non-finite temperature");
     }
     return ANISO_OK;
+}
+
+static int check_err3(aniso3_ctx *h)
+{
+    unsigned flag = 0;
+    CU(cudaMemcpy(&flag, h->err, sizeof flag, cudaMemcpyDeviceToHost));
+    return report_err3(h, flag);
 }
 
 extern "C" int aniso3_total(aniso3_t h, const void *T, double *sum, double *tmin, double *tmax,
@@ -257,15 +262,15 @@ extern "C" int aniso3_total(aniso3_t h, const void *T, double *sum, double *tmin
     if (!h) return fail(ANISO_ERR_ARG, "aniso3_total: null handle");
     if (!h->field_set) return fail(ANISO_ERR_STATE, "aniso3_total: call aniso3_set_field first");
     if (!T) return fail(ANISO_ERR_ARG, "aniso3_total: T is NULL");
-    CU(launch_totals(h->prec, T, h->cells(), h->partials, h->result, h->stream));
-    double r[4];
+    CU(launch_totals(h->prec, T, h->cells(), h->partials, h->result, h->stream, h->err));
+    double r[TOTALS_RESULT];
     CU(cudaMemcpyAsync(r, h->result, sizeof r, cudaMemcpyDeviceToHost, h->stream));
     CU(cudaStreamSynchronize(h->stream));
     if (sum) *sum = r[0];
     if (tmin) *tmin = r[1];
     if (tmax) *tmax = r[2];
     if (nonfinite) *nonfinite = (long long)r[3];
-    return check_err3(h);
+    return report_err3(h, (unsigned)r[4]);
 }
 
 extern "C" int aniso3_sync(aniso3_t h)

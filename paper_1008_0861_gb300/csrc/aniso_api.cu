@@ -346,7 +346,7 @@ extern "C" int aniso_set_field(aniso_t h, const void *bx, const void *by)
             }
         }
         CU(cudaMalloc(&h->partials, 4 * TOTALS_BLOCKS * sizeof(double)));
-        CU(cudaMalloc(&h->result, 4 * sizeof(double)));
+        CU(cudaMalloc(&h->result, TOTALS_RESULT * sizeof(double)));
         CU(cudaMalloc(&h->err, sizeof(unsigned)));
         CU(cudaMemsetAsync(h->err, 0, sizeof(unsigned), h->stream));
     }
@@ -934,10 +934,8 @@ extern "C" int aniso_sweep(aniso_t h, int dir, const void *Tin, void *Tout, doub
     return enqueue_sweep(h, dir, Tin, Tout, dt, h->stream, nullptr);
 }
 
-static int check_err_flag(aniso_ctx *h)
+static int report_err_flag(aniso_ctx *h, unsigned flag)
 {
-    unsigned flag = 0;
-    CU(cudaMemcpy(&flag, h->err, sizeof flag, cudaMemcpyDeviceToHost));
     if (flag) {
         CU(cudaMemset(h->err, 0, sizeof(unsigned)));
         if (flag & 2u) return fail(ANISO_ERR_TIMEOUT, "a kernel gave up waiting for its staged rows");
@@ -946,21 +944,29 @@ static int check_err_flag(aniso_ctx *h)
     return ANISO_OK;
 }
 
+static int check_err_flag(aniso_ctx *h)
+{
+    unsigned flag = 0;
+    CU(cudaMemcpy(&flag, h->err, sizeof flag, cudaMemcpyDeviceToHost));
+    return report_err_flag(h, flag);
+}
+
 extern "C" int aniso_total(aniso_t h, const void *T, double *sum, double *tmin, double *tmax,
                            long long *nonfinite)
 {
     int rc = check_ready(h, "aniso_total");
     if (rc) return rc;
     if (!T) return fail(ANISO_ERR_ARG, "aniso_total: T is NULL");
-    CU(launch_totals(h->prec, T, h->cells(), h->partials, h->result, h->stream, h->kahan ? h->tlo : nullptr));
-    double r[4];
+    CU(launch_totals(h->prec, T, h->cells(), h->partials, h->result, h->stream, h->err,
+                     h->kahan ? h->tlo : nullptr));
+    double r[TOTALS_RESULT];
     CU(cudaMemcpyAsync(r, h->result, sizeof r, cudaMemcpyDeviceToHost, h->stream));
     CU(cudaStreamSynchronize(h->stream));
     if (sum) *sum = r[0];
     if (tmin) *tmin = r[1];
     if (tmax) *tmax = r[2];
     if (nonfinite) *nonfinite = (long long)r[3];
-    return check_err_flag(h);
+    return report_err_flag(h, (unsigned)r[4]);
 }
 
 extern "C" int aniso_get_state(aniso_t h, long long *step_counter, void *lo_out)

@@ -235,20 +235,22 @@ cudaError_t launch_col(int prec, int coef_fp16, const ColArgs &a, int nblocks, i
                        size_t smem, cudaStream_t s, bool kahan = false);
 cudaError_t launch_line2(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads,
                          size_t smem, cudaStream_t s, bool kahan = false);
-// Face coefficients from cell-centred b (FP64 arithmetic, one rounding to the
-// storage type).  bprec: element type of bx, by.  coef: 0 fp64, 1 fp32, 2 fp16.
-// cyyT/cyxT (optional) receive transposed copies [nx][ny].
+// Face coefficients from cell-centred b (one rounding to the storage type).
+// bprec: element type of bx, by.  coef: 0 fp64, 1 fp32, 2 fp16.  cyy/cyx and
+// the transposed copies cyyT/cyxT [nx][ny] are each optional (null).
 cudaError_t launch_face_coeffs(int bprec, int coef, const void *bx, const void *by, int nx, int ny,
                                int bc, double kappa, void *cxx, void *cxy, void *cyy, void *cyx,
                                void *cyyT, void *cyxT, cudaStream_t s);
 // out[c][r] = in[r][c] for an rows x cols array of 4- or 8-byte elements.
 cudaError_t launch_transpose(int elem_bytes, const void *in, void *out, int rows, int cols,
                              cudaStream_t s);
-// FP64 sum / min / max / non-finite count; partial buffers of TOTALS_BLOCKS.
+// FP64 sum / min / max / non-finite count and the error word *err, as five
+// doubles in result; partial buffers of 4 x TOTALS_BLOCKS.
 constexpr int TOTALS_BLOCKS = 608;
+constexpr int TOTALS_RESULT = 5;
 // Tlo (optional, FP32): compensated low parts added to T in the sum.
 cudaError_t launch_totals(int prec, const void *T, size_t n, double *partials, double *result,
-                          cudaStream_t s, const void *Tlo = nullptr);
+                          cudaStream_t s, const unsigned *err, const void *Tlo = nullptr);
 
 // Set the message aniso_last_error() returns on this host thread.
 void record_error(const char *msg);

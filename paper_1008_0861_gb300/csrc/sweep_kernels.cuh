@@ -747,48 +747,129 @@ __global__ void __launch_bounds__(512) col_sweep_kernel(ColArgs args)
 
 // ======================================================= setup / utility
 
-// Face coefficients of Section 2 (b averaged to faces by the plain mean) in FP64
-// with explicit round-to-nearest operations (no contraction), then one
-// rounding to the storage type.
+// Face coefficients of Section 2 (b averaged to faces by the plain mean), one
+// rounding to the storage type: normal kappa + (1 - kappa) f_n^2, transverse
+// (1 - kappa) f_n f_t with f the mean of the two cells beside the face.
+//
+// From an FP64 field (or to FP64 storage) in FP64 with explicit
+// round-to-nearest operations (no contraction).  From an FP32 field to FP32 or
+// FP16 storage in double-word FP32 arithmetic (Dekker / Knuth: TwoSum, and the
+// product's error by fma), good to about 2^-46 before the one rounding: the
+// GPU does 2 FP64 operations a clock and SM, and their 18 a cell were most of
+// this kernel's time.  Components of 2^60 and more take the FP64 form (their
+// products could leave FP32's range where the coefficient does not).
 template <typename C> __device__ __forceinline__ C to_store(double v);
 template <> __device__ __forceinline__ double to_store<double>(double v) { return v; }
 template <> __device__ __forceinline__ float to_store<float>(double v) { return __double2float_rn(v); }
 template <> __device__ __forceinline__ __half to_store<__half>(double v) { return __double2half(v); }
 
-template <typename B, typename C>
-__global__ void face_coeffs_kernel(const B *__restrict__ bx, const B *__restrict__ by, int nx,
-                                   int ny, int bc, double kappa, C *cxx, C *cxy, C *cyy, C *cyx,
-                                   C *cyyT, C *cyxT)
+// s + t rounded once to the storage type (|t| at most about an ulp of s).
+template <typename C> __device__ __forceinline__ C to_store2(float s, float t);
+template <> __device__ __forceinline__ float to_store2<float>(float s, float t) { return __fadd_rn(s, t); }
+template <> __device__ __forceinline__ __half to_store2<__half>(float s, float t)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y;
-    if (i >= nx || j >= ny) return;
-    const size_t o = (size_t)j * nx + i;
+    // to FP32 by rounding to odd (an inexact sum gets an odd last bit), so that the rounding to FP16 is the only one
+    const float h = __fadd_rn(s, t), l = __fsub_rn(t, __fsub_rn(h, s));
+    unsigned b = __float_as_uint(h);
+    if (l != 0.f && (b & 1u) == 0u) b += ((__float_as_uint(l) ^ b) >> 31) ? ~0u : 1u;
+    return __float2half_rn(__uint_as_float(b));
+}
+
+struct Word2 {  // hi + lo
+    float h, l;
+};
+__device__ __forceinline__ Word2 mean2(float a, float b)
+{
+    const float s = __fadd_rn(a, b), c = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, c)), __fsub_rn(b, c));
+    return {0.5f * s, 0.5f * e};
+}
+// kap + omk (x y), kap and omk as pairs; kap = (0, 0) for the transverse coefficient
+__device__ __forceinline__ Word2 coef2(Word2 x, Word2 y, Word2 omk, Word2 kap)
+{
+    const float p = __fmul_rn(x.h, y.h);
+    const float e = __fmaf_rn(x.l, y.h, __fmaf_rn(x.h, y.l, __fmaf_rn(x.h, y.h, -p)));
+    const float q = __fmul_rn(p, omk.h);
+    const float r = __fmaf_rn(e, omk.h, __fmaf_rn(p, omk.l, __fmaf_rn(p, omk.h, -q)));
+    const float s = __fadd_rn(kap.h, q), c = __fsub_rn(s, kap.h);
+    const float t = __fadd_rn(__fsub_rn(kap.h, __fsub_rn(s, c)), __fsub_rn(q, c));
+    return {s, __fadd_rn(t, __fadd_rn(kap.l, r))};
+}
+
+// Both coefficients of one face: bn, bt the components along the face normal
+// and across it, in the cells before (0) and after (1) the face.
+template <typename B, typename C>
+__device__ __forceinline__ void face_coef(B bn0, B bn1, B bt0, B bt1, double kappa, C &cn, C &ct)
+{
+    if constexpr (sizeof(B) == 4 && sizeof(C) <= 4) {
+        const float big = fmaxf(fmaxf(fabsf(bn0), fabsf(bn1)), fmaxf(fabsf(bt0), fabsf(bt1)));
+        if (big < 0x1p60f) {
+            const double o = __dsub_rn(1.0, kappa);
+            Word2 omk, kap;
+            omk.h = __double2float_rn(o);
+            omk.l = __double2float_rn(__dsub_rn(o, (double)omk.h));
+            kap.h = __double2float_rn(kappa);
+            kap.l = __double2float_rn(__dsub_rn(kappa, (double)kap.h));
+            const Word2 fn = mean2(bn0, bn1), ft = mean2(bt0, bt1);
+            const Word2 n = coef2(fn, fn, omk, kap), t = coef2(fn, ft, omk, Word2{0.f, 0.f});
+            cn = to_store2<C>(n.h, n.l);
+            ct = to_store2<C>(t.h, t.l);
+            return;
+        }
+    }
     const double omk = __dsub_rn(1.0, kappa);
-    double vxx = 0.0, vxy = 0.0, vyy = 0.0, vyx = 0.0;
+    const double fn = __dmul_rn(0.5, __dadd_rn((double)bn0, (double)bn1));
+    const double ft = __dmul_rn(0.5, __dadd_rn((double)bt0, (double)bt1));
+    cn = to_store<C>(__dadd_rn(kappa, __dmul_rn(omk, __dmul_rn(fn, fn))));
+    ct = to_store<C>(__dmul_rn(omk, __dmul_rn(fn, ft)));
+}
+
+// One block a 32 x 32 tile of cells (32 x 8 threads).  The y faces' values go
+// out in the natural layout (cyy, cyx) and, where asked for (cyyT, cyxT),
+// through shared memory as whole rows of the transposed one: written by
+// column from the natural order, every 4-byte store was a sector of its own.
+// 1024^2 FP32: 64 us a call with both, 8 now.
+template <typename B, typename C>
+__global__ void __launch_bounds__(256) face_coeffs_kernel(const B *__restrict__ bx, const B *__restrict__ by, int nx,
+                                                          int ny, int bc, double kappa, C *cxx, C *cxy, C *cyy, C *cyx,
+                                                          C *cyyT, C *cyxT)
+{
+    __shared__ C tyy[32][33], tyx[32][33];
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
+    const int i = i0 + threadIdx.x;
     const bool per = bc == 1;  // otherwise the boundary faces carry no flux
-    if (per || i != nx - 1) {
-        const size_t o1 = (size_t)j * nx + ((i + 1) % nx);
-        const double fbx = __dmul_rn(0.5, __dadd_rn((double)bx[o], (double)bx[o1]));
-        const double fby = __dmul_rn(0.5, __dadd_rn((double)by[o], (double)by[o1]));
-        vxx = __dadd_rn(kappa, __dmul_rn(omk, __dmul_rn(fbx, fbx)));
-        vxy = __dmul_rn(omk, __dmul_rn(fbx, fby));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = threadIdx.y + 8 * k, j = j0 + r;
+        if (i < nx && j < ny) {
+            const size_t o = (size_t)j * nx + i;
+            const size_t ox = i + 1 < nx ? o + 1 : o - (nx - 1);
+            const size_t oy = j + 1 < ny ? o + nx : (size_t)i;
+            const B x0 = bx[o], y0 = by[o];
+            C vxx = C(0.f), vxy = C(0.f), vyy = C(0.f), vyx = C(0.f);
+            if (per || i != nx - 1) face_coef<B, C>(x0, bx[ox], y0, by[ox], kappa, vxx, vxy);
+            if (per || j != ny - 1) face_coef<B, C>(y0, by[oy], x0, bx[oy], kappa, vyy, vyx);
+            cxx[o] = vxx;
+            cxy[o] = vxy;
+            if (cyy) {
+                cyy[o] = vyy;
+                cyx[o] = vyx;
+            }
+            tyy[r][threadIdx.x] = vyy;
+            tyx[r][threadIdx.x] = vyx;
+        }
     }
-    if (per || j != ny - 1) {
-        const size_t o1 = (size_t)((j + 1) % ny) * nx + i;
-        const double fbx = __dmul_rn(0.5, __dadd_rn((double)bx[o], (double)bx[o1]));
-        const double fby = __dmul_rn(0.5, __dadd_rn((double)by[o], (double)by[o1]));
-        vyy = __dadd_rn(kappa, __dmul_rn(omk, __dmul_rn(fby, fby)));
-        vyx = __dmul_rn(omk, __dmul_rn(fby, fbx));
-    }
-    cxx[o] = to_store<C>(vxx);
-    cxy[o] = to_store<C>(vxy);
-    cyy[o] = to_store<C>(vyy);
-    cyx[o] = to_store<C>(vyx);
-    if (cyyT) {
-        const size_t oT = (size_t)i * ny + j;
-        cyyT[oT] = to_store<C>(vyy);
-        cyxT[oT] = to_store<C>(vyx);
+    if (!cyyT) return;
+    __syncthreads();
+    const int j = j0 + threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = threadIdx.y + 8 * k;
+        if (i0 + c < nx && j < ny) {
+            const size_t oT = (size_t)(i0 + c) * ny + j;
+            cyyT[oT] = tyy[threadIdx.x][c];
+            cyxT[oT] = tyx[threadIdx.x][c];
+        }
     }
 }
 
@@ -808,62 +889,103 @@ __global__ void transpose_kernel(const E *__restrict__ in, E *__restrict__ out, 
     }
 }
 
-// Deterministic FP64 reductions: a fixed grid of TOTALS_BLOCKS blocks, each
-// thread a fixed strided subset, fixed-order trees.
+// Deterministic reductions: a fixed grid of TOTALS_BLOCKS blocks, each thread
+// a fixed strided subset, fixed-order trees.  The sum is formed in FP64; the
+// extrema are compared as integers (sign-magnitude bits made monotonic) and
+// non-finite values told by their exponent, so that FP64 data cost one FP64
+// operation a value.
+__device__ __forceinline__ long long order_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double from_key(long long k)
+{
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
+constexpr long long KEY_PINF = 0x7ff0000000000000ll, KEY_MINF = ~0x7ff0000000000000ll;  // keys of +-infinity
+
+struct Totals {
+    double s;
+    long long lo, hi, nf;
+    __device__ __forceinline__ void add(const Totals &o)
+    {
+        s += o.s;
+        lo = o.lo < lo ? o.lo : lo;
+        hi = o.hi > hi ? o.hi : hi;
+        nf += o.nf;
+    }
+};
+// The block's total in thread 0: warps by shuffles, then warp 0 (a fixed order).
+__device__ __forceinline__ Totals totals_block(Totals t)
+{
+    __shared__ Totals part[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto warp_sum = [](Totals &v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            Totals w;
+            w.s = __shfl_down_sync(0xffffffffu, v.s, o);
+            w.lo = __shfl_down_sync(0xffffffffu, v.lo, o);
+            w.hi = __shfl_down_sync(0xffffffffu, v.hi, o);
+            w.nf = __shfl_down_sync(0xffffffffu, v.nf, o);
+            v.add(w);
+        }
+    };
+    warp_sum(t);
+    if (lane == 0) part[warp] = t;
+    __syncthreads();
+    if (warp == 0) {
+        t = lane < (int)(blockDim.x >> 5) ? part[lane] : Totals{0.0, KEY_PINF, KEY_MINF, 0};
+        warp_sum(t);
+    }
+    return t;
+}
+
 template <typename R>
 __global__ void __launch_bounds__(256) totals_partial_kernel(const R *__restrict__ T, const R *__restrict__ Tlo,
                                                              size_t n, double *partials)
 {
-    __shared__ double ss[256], smin[256], smax[256], snf[256];
-    double s = 0.0, lo = INFINITY, hi = -INFINITY, nf = 0.0;
+    Totals t{0.0, KEY_PINF, KEY_MINF, 0};
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
         const double v = Tlo ? (double)T[k] + (double)Tlo[k] : (double)T[k];
-        if (isfinite(v)) {
-            s += v;
-            lo = fmin(lo, v);
-            hi = fmax(hi, v);
+        const long long key = order_key(v);
+        if (key < KEY_PINF && key > KEY_MINF) {
+            t.s += v;
+            t.lo = key < t.lo ? key : t.lo;
+            t.hi = key > t.hi ? key : t.hi;
         } else {
-            nf += 1.0;
+            t.nf += 1;
         }
     }
-    ss[threadIdx.x] = s;
-    smin[threadIdx.x] = lo;
-    smax[threadIdx.x] = hi;
-    snf[threadIdx.x] = nf;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if (threadIdx.x < h) {
-            ss[threadIdx.x] += ss[threadIdx.x + h];
-            smin[threadIdx.x] = fmin(smin[threadIdx.x], smin[threadIdx.x + h]);
-            smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + h]);
-            snf[threadIdx.x] += snf[threadIdx.x + h];
-        }
-        __syncthreads();
-    }
+    t = totals_block(t);
     if (threadIdx.x == 0) {
-        partials[blockIdx.x] = ss[0];
-        partials[gridDim.x + blockIdx.x] = smin[0];
-        partials[2 * gridDim.x + blockIdx.x] = smax[0];
-        partials[3 * gridDim.x + blockIdx.x] = snf[0];
+        partials[blockIdx.x] = t.s;
+        partials[gridDim.x + blockIdx.x] = from_key(t.lo);
+        partials[2 * gridDim.x + blockIdx.x] = from_key(t.hi);
+        partials[3 * gridDim.x + blockIdx.x] = (double)t.nf;
     }
 }
 
-static __global__ void __launch_bounds__(32) totals_final_kernel(const double *partials, int nb,
-                                                          double *result)
+// The blocks' partials in one block (one thread reading all of them in turn
+// took 138 us), and the step's error word beside them, so that the host takes
+// everything in one copy.
+static __global__ void __launch_bounds__(256) totals_final_kernel(const double *partials, int nb, const unsigned *err,
+                                                                  double *result)
 {
-    if (threadIdx.x != 0) return;
-    double s = 0.0, lo = INFINITY, hi = -INFINITY, nf = 0.0;
-    for (int b = 0; b < nb; ++b) {
-        s += partials[b];
-        lo = fmin(lo, partials[nb + b]);
-        hi = fmax(hi, partials[2 * nb + b]);
-        nf += partials[3 * nb + b];
+    Totals t{0.0, KEY_PINF, KEY_MINF, 0};
+    for (int b = threadIdx.x; b < nb; b += blockDim.x)
+        t.add(Totals{partials[b], order_key(partials[nb + b]), order_key(partials[2 * nb + b]),
+                     (long long)partials[3 * nb + b]});
+    t = totals_block(t);
+    if (threadIdx.x == 0) {
+        result[0] = t.s;
+        result[1] = from_key(t.lo);
+        result[2] = from_key(t.hi);
+        result[3] = (double)t.nf;
+        result[4] = (double)*err;
     }
-    result[0] = s;
-    result[1] = lo;
-    result[2] = hi;
-    result[3] = nf;
 }
 
 }  // namespace aniso

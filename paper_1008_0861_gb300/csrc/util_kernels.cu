@@ -245,7 +245,7 @@ template <typename B, typename C>
 static void face_launch(const void *bx, const void *by, int nx, int ny, int bc, double kappa, void *cxx,
                         void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s)
 {
-    dim3 block(256), grid((nx + 255) / 256, ny);
+    dim3 block(32, 8), grid((nx + 31) / 32, (ny + 31) / 32);
     face_coeffs_kernel<B, C><<<grid, block, 0, s>>>(
         static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, kappa, static_cast<C *>(cxx),
         static_cast<C *>(cxy), static_cast<C *>(cyy), static_cast<C *>(cyx), static_cast<C *>(cyyT),
@@ -282,7 +282,7 @@ cudaError_t launch_transpose(int elem_bytes, const void *in, void *out, int rows
 }
 
 cudaError_t launch_totals(int prec, const void *T, size_t n, double *partials, double *result,
-                          cudaStream_t s, const void *Tlo)
+                          cudaStream_t s, const unsigned *err, const void *Tlo)
 {
     if (prec == PREC_FP64)
         totals_partial_kernel<double><<<TOTALS_BLOCKS, 256, 0, s>>>(static_cast<const double *>(T), nullptr, n,
@@ -290,7 +290,7 @@ cudaError_t launch_totals(int prec, const void *T, size_t n, double *partials, d
     else
         totals_partial_kernel<float><<<TOTALS_BLOCKS, 256, 0, s>>>(static_cast<const float *>(T),
                                                                    static_cast<const float *>(Tlo), n, partials);
-    totals_final_kernel<<<1, 32, 0, s>>>(partials, TOTALS_BLOCKS, result);
+    totals_final_kernel<<<1, 256, 0, s>>>(partials, TOTALS_BLOCKS, err, result);
     return cudaGetLastError();
 }
 
