@@ -169,8 +169,9 @@ extern "C" int aniso3_set_field(aniso3_t h, const void *bx, const void *by, cons
 
 // One update along axis d (0 x, 1 y, 2 z) of lines laid out for that axis:
 // transverse axes a = d+1, b = d+2 (cyclic), line index kb * n[a] + ka.
+// chained: the launch before is one of the same call's.
 static int enqueue3(aniso3_ctx *h, int d, const void *in, void *out, double lam, double mua, double mub,
-                    bool transposed)
+                    bool transposed, bool chained)
 {
     const int a = (d + 1) % 3, b = (d + 2) % 3;
     Line2Args A{};
@@ -178,6 +179,7 @@ static int enqueue3(aniso3_ctx *h, int d, const void *in, void *out, double lam,
     A.njobs = 1;
     A.limiter = h->limiter;
     A.err = h->err;
+    A.chained = chained;
     Line2Job &J = A.one;
     J.Tin = in;
     J.Tout = out;
@@ -223,18 +225,18 @@ extern "C" int aniso3_step(aniso3_t h, void *T, double dt, int nsteps)
     for (int s = 0; s < nsteps; ++s) {
         if (h->scheme == ANISO_SCHEME_2STEP) {
             // T [z][y][x] -> s1 [x][z][y] -> s2 [y][x][z] -> T [z][y][x]
-            if ((rc = enqueue3(h, 0, T, h->s1, lam[0], mu[0], mu[1], true))) return rc;
-            if ((rc = enqueue3(h, 1, h->s1, h->s2, lam[1], mu[2], mu[3], true))) return rc;
-            if ((rc = enqueue3(h, 2, h->s2, T, lam[2], mu[4], mu[5], true))) return rc;
+            if ((rc = enqueue3(h, 0, T, h->s1, lam[0], mu[0], mu[1], true, s > 0))) return rc;
+            if ((rc = enqueue3(h, 1, h->s1, h->s2, lam[1], mu[2], mu[3], true, true))) return rc;
+            if ((rc = enqueue3(h, 2, h->s2, T, lam[2], mu[4], mu[5], true, true))) return rc;
         } else {
             // per axis: half-coefficient update with the transverse terms
             // (same layout), then a purely implicit half update (transposed)
-            if ((rc = enqueue3(h, 0, T, h->s1, 0.5 * lam[0], mu[0], mu[1], false))) return rc;
-            if ((rc = enqueue3(h, 0, h->s1, h->s2, 0.5 * lam[0], 0.0, 0.0, true))) return rc;
-            if ((rc = enqueue3(h, 1, h->s2, h->s1, 0.5 * lam[1], mu[2], mu[3], false))) return rc;
-            if ((rc = enqueue3(h, 1, h->s1, h->s2, 0.5 * lam[1], 0.0, 0.0, true))) return rc;
-            if ((rc = enqueue3(h, 2, h->s2, h->s1, 0.5 * lam[2], mu[4], mu[5], false))) return rc;
-            if ((rc = enqueue3(h, 2, h->s1, T, 0.5 * lam[2], 0.0, 0.0, true))) return rc;
+            if ((rc = enqueue3(h, 0, T, h->s1, 0.5 * lam[0], mu[0], mu[1], false, s > 0))) return rc;
+            if ((rc = enqueue3(h, 0, h->s1, h->s2, 0.5 * lam[0], 0.0, 0.0, true, true))) return rc;
+            if ((rc = enqueue3(h, 1, h->s2, h->s1, 0.5 * lam[1], mu[2], mu[3], false, true))) return rc;
+            if ((rc = enqueue3(h, 1, h->s1, h->s2, 0.5 * lam[1], 0.0, 0.0, true, true))) return rc;
+            if ((rc = enqueue3(h, 2, h->s2, h->s1, 0.5 * lam[2], mu[4], mu[5], false, true))) return rc;
+            if ((rc = enqueue3(h, 2, h->s1, T, 0.5 * lam[2], 0.0, 0.0, true, true))) return rc;
         }
     }
     return ANISO_OK;

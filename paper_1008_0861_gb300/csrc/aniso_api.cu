@@ -94,6 +94,9 @@ struct aniso_ctx {
     int tmem = 1;       // ANISO_OPT_TMEM
     int cluster = 2;    // ANISO_OPT_CLUSTER_LINES
     double nl_alpha = 0, nl_tref = 1;  // temperature-dependent diffusivity (aniso_set_nonlinear)
+    // the launch before in this call was one of this handle's kernels, so the
+    // next line kernel may be launched to overlap its end
+    bool chained = false;
     void *t4 = nullptr;  // intermediate of the 4-step scheme
     void *q = nullptr;   // source term (aniso_set_source), handle precision
     cudaStream_t stream = 0;
@@ -420,6 +423,8 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     if (!ok) return fail(ANISO_ERR_UNSUPPORTED, "vectorised line kernel cannot take n=%d", n);
     J.block0 = 0;
     J.nblocks = (nlines + J.lines_per_block - 1) / J.lines_per_block;
+    a.chained = h->chained && !h->profile && !v7;  // (a timing event between two launches keeps them apart)
+    h->chained = true;
     int pidx = -1;
     const unsigned rec_flags = pairs ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (h->profile) {
@@ -700,6 +705,7 @@ static int enqueue_steps_any_order(aniso_ctx *h, void *T, double dt, int nsteps,
 static int enqueue_steps(aniso_ctx *h, void *T, double dt, int nsteps, long long counter0,
                          cudaStream_t s, std::vector<int> *pairs)
 {
+    h->chained = false;
     if (h->scheme == ANISO_SCHEME_EXPLICIT) {
         // explicit limited steps, T -> T* -> T ...; an odd count ends with a copy back
         ExpArgs a{};
@@ -931,6 +937,7 @@ extern "C" int aniso_sweep(aniso_t h, int dir, const void *Tin, void *Tout, doub
     if (!(dt > 0)) return fail(ANISO_ERR_ARG, "aniso_sweep: dt must be > 0");
     if (h->nl_alpha != 0.0)
         return fail(ANISO_ERR_UNSUPPORTED, "aniso_sweep: not with the temperature-dependent diffusivity");
+    h->chained = false;
     return enqueue_sweep(h, dir, Tin, Tout, dt, h->stream, nullptr);
 }
 
@@ -1638,6 +1645,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             aniso_ctx *h = b->hs[L.inst];
             const int saved = h->profile;  // these sweeps are not profiled inside the batch
             h->profile = 0;
+            h->chained = false;  // (other grids' launches lie between)
             rc = L.kind == 13 ? enqueue_fast_sweep(h, L.dir, L.out, L.dt, b->cap_stream, nullptr)
                               : enqueue_sweep(h, L.dir, L.in, L.out, L.dt, b->cap_stream, nullptr, L.in_lo, L.out_lo);
             h->profile = saved;

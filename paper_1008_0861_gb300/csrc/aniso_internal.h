@@ -132,6 +132,9 @@ struct Line2Args {
     // line4, FP32 2-D, four-warp blocks: 1 keeps each lane's gamma in tensor
     // memory (the launch's shared memory then holds two arrays, not three)
     int tmem;
+    // 1: launched to start while the kernel before it in the stream drains
+    // (programmatic dependent launch); never the first launch of a captured call
+    int chained;
 };
 // Finish the diagnostics of one line4 launch: for every job, the partials of
 // its blocks in block order -> ring[diag_slot] = (sum, min, max).

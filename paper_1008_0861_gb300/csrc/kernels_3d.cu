@@ -101,8 +101,7 @@ template <typename K> static cudaError_t run4_3d(K kern, const Line2Args &a, int
                 cudaSuccess)
             return e;
     }
-    kern<<<nblocks, nthreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
 }
 
 cudaError_t launch_line4_3d(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,

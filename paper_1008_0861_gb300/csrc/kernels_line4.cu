@@ -16,8 +16,7 @@ template <typename K> static cudaError_t run4(K kern, const Line2Args &a, int nb
                 cudaSuccess)
             return e;
     }
-    kern<<<nblocks, nthreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
 }
 
 cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,

@@ -39,8 +39,7 @@ template <typename K> static cudaError_t run6(K kern, const Line2Args &a, int nb
     if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
-    kern<<<nblocks, nthreads, smem, s>>>(a);
-    return cudaGetLastError();
+    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
 }
 
 cudaError_t launch_line6(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)

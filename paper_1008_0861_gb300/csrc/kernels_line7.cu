@@ -32,19 +32,8 @@ static cudaError_t run7(Kern kern, const Line2Args &a, int cs, size_t smem, cuda
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     const int groups = (a.one.nlines + L7_LPB - 1) / L7_LPB;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(groups * cs), 1, 1);
-    cfg.blockDim = dim3(L7_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cs;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    // (a is never chained here: launches of 100 us and more gain nothing, 4096^2 lost 0.4 %)
+    return launch_line_kernel(kern, a, groups * cs, L7_THREADS, smem, s, cs);
 }
 
 template <bool K, bool TM, bool TO>

@@ -67,6 +67,44 @@ __device__ __forceinline__ void l2_prefetch(const void *p, size_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"((unsigned)bytes) : "memory");
 }
 
+// Programmatic dependent launch: a kernel launched with args.chained may start
+// while the one before it in the stream still runs.  It waits here, before it
+// first touches memory the other writes, and then lets the next one start.
+// (Both are no-ops in a plain launch.)
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// Host: a launch of kern(a) in a.chained mode or plainly.
+template <typename K>
+static cudaError_t launch_line_kernel(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s,
+                                      int cluster = 0)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblocks, 1, 1);
+    cfg.blockDim = dim3((unsigned)nthreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if (cluster > 0) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = (unsigned)cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (a.chained) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
 __device__ __forceinline__ float frcp_approx(float x)
 {
     float r;
@@ -401,6 +439,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
     const R chi_a = (R)J.chi_alpha, chi_it = (R)J.chi_itref;
     auto chi_of = [chi_a, chi_it](R T_) { return T_ > R(0) ? chi_pow<R>(T_ * chi_it, chi_a) : R(0); };
     const unsigned full = 0xffffffffu;
+
+    // (what came before is the kernel's own arguments and indices)
+    chain_wait();
 
     // The block's input rows (its lines and the two neighbouring lines of T,
     // its coefficient rows) start streaming into L2 at once, so that the
