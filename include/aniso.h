@@ -86,7 +86,8 @@ enum {
     ANISO_OPT_SEGMENT = 9,    /* cells per thread segment of the vectorised kernels, in 16-byte
                                  chunks (0 = default: 4, fewer for a small FP64 grid stepped alone;
                                  larger: fewer threads per line and so a shallower PCR) */
-    ANISO_OPT_BLOCK_WARPS = 10, /* warps per block of the warp-autonomous kernel (0 = default 4;
+    ANISO_OPT_BLOCK_WARPS = 10, /* warps per block of the warp-autonomous kernel (0 = default: 4, 8 for
+                                   middling FP32 grids stepped alone;
                                    1, 2, 4 or 8): lines per block = warps x lines per warp */
     ANISO_OPT_SCHEME = 11,     /* ANISO_SCHEME_2STEP (default), _4STEP or _EXPLICIT; the other
                                   schemes run on single handles (aniso_step, not batches) with

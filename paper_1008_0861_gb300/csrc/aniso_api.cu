@@ -397,7 +397,10 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     int nthreads;
     size_t smem;
     const int seg = v4 && h->seg_chunks == 0 && h->prec == PREC_FP64 ? line4_seg_fp64(n, nlines) : h->seg_chunks;
-    bool ok = v4 ? line4_config(h->prec, n, transposed, h->l4_warps, seg, &J.team, &J.lines_per_block, &nthreads,
+    const int warps = v4 && transposed && h->l4_warps == 0 && h->seg_chunks == 0 && h->prec == PREC_FP32
+                          ? line4_warps_alone(n, nlines)
+                          : h->l4_warps;
+    bool ok = v4 ? line4_config(h->prec, n, transposed, warps, seg, &J.team, &J.lines_per_block, &nthreads,
                                 &smem)
                  : line2_config(h->prec, n, transposed, &J.team, &J.lines_per_block, &nthreads, &smem,
                                 h->seg_chunks);

@@ -23,6 +23,11 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
                          cudaStream_t s)
 {
     const bool vl = a.limiter == LIM_VANLEER;
+    // A grid alone that leaves an SM at most 16 warps (of the 32 the 64-register
+    // form allows) waits for its loads: three rounds in flight in the 128-register
+    // form.  FP32 us an update, one round / three: 128^2 4.68 / 4.27, 512^2
+    // 5.34 / 4.63, 768^2 8.21 / 7.55, 1024^2 10.4 / 10.2, 1536^2 (16 warps) 16.9 / 17.1
+    const bool deep = !a.jobs && (long)nblocks * nthreads <= 152L * 32 * 8;
     if (!a.jobs && a.one.mu == 0.0 && a.one.chi_alpha == 0.0) {  // purely implicit update (4-step halves)
         if (prec == PREC_FP64)
             return run4(line4_kernel<double, double, false, false, false, true>, a, nblocks, nthreads, smem, s);
@@ -35,6 +40,8 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
         if (prec == PREC_FP64)
             return vl ? run4(line4_kernel<double, double, true, false, true>, a, nblocks, nthreads, smem, s)
                       : run4(line4_kernel<double, double, false, false, true>, a, nblocks, nthreads, smem, s);
+        if (vl && deep)
+            return run4(line4_kernel<float, float, true, false, true, false, false, 3>, a, nblocks, nthreads, smem, s);
         return vl ? run4(line4_kernel<float, float, true, false, true>, a, nblocks, nthreads, smem, s)
                   : run4(line4_kernel<float, float, false, false, true>, a, nblocks, nthreads, smem, s);
     }
@@ -48,6 +55,9 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
     if (prec == PREC_FP64)
         return vl ? run4(line4_kernel<double, double, true>, a, nblocks, nthreads, smem, s)
                   : run4(line4_kernel<double, double, false>, a, nblocks, nthreads, smem, s);
+    if (vl && deep)
+        return coef_fp16 ? run4(line4_kernel<float, __half, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s)
+                         : run4(line4_kernel<float, float, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s);
     if (coef_fp16)
         return vl ? run4(line4_kernel<float, __half, true>, a, nblocks, nthreads, smem, s)
                   : run4(line4_kernel<float, __half, false>, a, nblocks, nthreads, smem, s);
@@ -102,6 +112,21 @@ int line4_seg_fp64(int n, int nlines)
         }
     }
     return best;
+}
+
+// Warps a block for one FP32 grid's update on its own.  Lines of 512 cells and
+// more (one a warp) leave a four-warp block four lines wide, so its transposed
+// store writes half sectors; eight warps write whole ones.  That is taken where
+// eight-warp blocks fill most SMs and run in one wave (768^2: 7.55 -> 7.26 us an
+// update, 1024^2: 10.2 -> 9.4; 512^2, 64 blocks: 4.63 -> 5.37; 1280^2, a second
+// wave: 13.9 -> 20.4).
+int line4_warps_alone(int n, int nlines)
+{
+    int team, lpb, nt;
+    size_t smem;
+    if (!line4_config(PREC_FP32, n, true, 8, 0, &team, &lpb, &nt, &smem) || lpb != 8 || nt != 256) return 0;
+    const long blocks = ((long)nlines + 7) / 8, resident = (long)((SMEM_LIMIT - 1024) / (smem + 1024));
+    return blocks >= 96 && blocks <= 152 * (resident < 4 ? resident : 4) ? 8 : 0;
 }
 
 // The kernel keeps 16-byte chunk c of a line at c ^ ((c >> s) & 7) inside

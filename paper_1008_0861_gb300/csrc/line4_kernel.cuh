@@ -213,6 +213,13 @@ template <> struct Limit<double, true, true> {
     }
 };
 
+// Which product of a flux is fused with the sum is spelled out, so that every
+// form of the kernel rounds alike (a batch equals its grids one by one).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // NaN or infinity (the exponent bits, off the FP64 pipe).
 __device__ __forceinline__ bool non_finite(float v) { return !(fabsf(v) < INFINITY); }
 __device__ __forceinline__ bool non_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
@@ -385,8 +392,9 @@ __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sy
 // shared memory is 8 bytes a cell instead of 12 and more blocks fit an SM; the
 // lane's chunks of T_old wait there too, from the flux phase to phase C
 // (4 V + 4 V columns of the block's 32 or 64).
-template <typename R, typename C, bool VL, bool D3 = false, bool NL = false, bool IMPL = false, bool TM = false>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_kernel(Line2Args args)
+template <typename R, typename C, bool VL, bool D3 = false, bool NL = false, bool IMPL = false, bool TM = false,
+          int RING = 1>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4) : 2) line4_kernel(Line2Args args)
 {
     static_assert(!TM || (sizeof(R) == 4 && !D3), "TMEM line state: FP32 2-D only");
     typedef typename V16<R>::T VT;
@@ -440,8 +448,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
     auto chi_of = [chi_a, chi_it](R T_) { return T_ > R(0) ? chi_pow<R>(T_ * chi_it, chi_a) : R(0); };
     const unsigned full = 0xffffffffu;
 
-    // (what came before is the kernel's own arguments and indices)
-    chain_wait();
+    // (what came before is the kernel's own arguments and indices; batched
+    // launches, the only ones in the tensor-memory form, are never chained)
+    if (!TM && !args.jobs) chain_wait();
 
     // The block's input rows (its lines and the two neighbouring lines of T,
     // its coefficient rows) start streaming into L2 at once, so that the
@@ -497,21 +506,26 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
         const VT *vbd = reinterpret_cast<const VT *>(rbd), *vbu = reinterpret_cast<const VT *>(rbu);
         R Tcar = R(0), vcar = R(0);  // cell 0 of chunk (v+1)P, from the team's lane 0
         R wcar = R(0);               // the same for the second transverse axis (D3)
-        // the next round's loads are issued before this round's arithmetic
-        int cl = min(((V - 1) << logP) + t, m - 1);
-        VT xc = vc[cl], xd = xc, xu = xc;
-        auto xg = ld_raw(G + cl * N), xe = xg;
-        if constexpr (!IMPL) {
-            xd = vd[cl];
-            xu = vu[cl];
-            xe = ld_raw(E + cl * N);
-        }
-        VT xbd = xc, xbu = xc;
-        auto xe2 = xe;
-        if constexpr (D3 && !IMPL) {
-            xbd = vbd[cl];
-            xbu = vbu[cl];
-            xe2 = ld_raw(E2 + cl * N);
+        // the loads of the next RING rounds are issued before a round's arithmetic
+        typedef decltype(ld_raw(G)) CT;
+        int cl[RING];
+        VT xc[RING], xd[RING], xu[RING], xbd[RING], xbu[RING];
+        CT xg[RING], xe[RING], xe2[RING];
+#pragma unroll
+        for (int r = 0; r < RING; ++r) {
+            cl[r] = min((max(V - 1 - r, 0) << logP) + t, m - 1);
+            xc[r] = xd[r] = xu[r] = xbd[r] = xbu[r] = vc[cl[r]];
+            xg[r] = xe[r] = xe2[r] = ld_raw(G + cl[r] * N);
+            if constexpr (!IMPL) {
+                xd[r] = vd[cl[r]];
+                xu[r] = vu[cl[r]];
+                xe[r] = ld_raw(E + cl[r] * N);
+            }
+            if constexpr (D3 && !IMPL) {
+                xbd[r] = vbd[cl[r]];
+                xbu[r] = vbu[cl[r]];
+                xe2[r] = ld_raw(E2 + cl[r] * N);
+            }
         }
         // the cell after the line (periodic wrap or mirrored ghost), issued
         // with the first round's loads instead of inside that round (2-D; the
@@ -533,38 +547,42 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
             tm_base = s_tmem;
             tm_lane = tm_base + ((unsigned)(32 * (warp & 3)) << 16);
         }
-        for (int v = V - 1; v >= 0; --v) {
+        for (int v0 = V - 1; v0 >= 0; v0 -= RING)
+#pragma unroll
+        for (int r = 0; r < RING; ++r) {
+            const int v = v0 - r;
+            if (RING > 1 && v < 0) break;
             const int c = (v << logP) + t;
             R Td[N], Tc[N], Tu[N], Gv[N], Ev[N], Tbd[N], Tbu[N], E2v[N];
-            V16<R>::unpack(xc, Tc);
+            V16<R>::unpack(xc[r], Tc);
             // TMEM form: this chunk of T_old waits in the lane's columns 4 (V + v)
             // for phase C, which takes the same chunks by the same lanes
             if constexpr (TM) tm_st4(tm_lane + 4u * (unsigned)(V + v), Tc[0], Tc[1], Tc[2], Tc[3]);
-            unpack_raw(xg, Gv);
+            unpack_raw(xg[r], Gv);
             if constexpr (!IMPL) {
-                V16<R>::unpack(xd, Td);
-                V16<R>::unpack(xu, Tu);
-                unpack_raw(xe, Ev);
+                V16<R>::unpack(xd[r], Td);
+                V16<R>::unpack(xu[r], Tu);
+                unpack_raw(xe[r], Ev);
             }
             if constexpr (D3 && !IMPL) {
-                V16<R>::unpack(xbd, Tbd);
-                V16<R>::unpack(xbu, Tbu);
-                unpack_raw(xe2, E2v);
+                V16<R>::unpack(xbd[r], Tbd);
+                V16<R>::unpack(xbu[r], Tbu);
+                unpack_raw(xe2[r], E2v);
             }
-            const int cur = cl;
-            if (v > 0) {
-                cl = ((v - 1) << logP) + t;  // always < m
-                xc = vc[cl];
-                xg = ld_raw(G + cl * N);
+            const int cur = cl[r];
+            if (v >= RING) {
+                cl[r] = ((v - RING) << logP) + t;  // always < m
+                xc[r] = vc[cl[r]];
+                xg[r] = ld_raw(G + cl[r] * N);
                 if constexpr (!IMPL) {
-                    xd = vd[cl];
-                    xu = vu[cl];
-                    xe = ld_raw(E + cl * N);
+                    xd[r] = vd[cl[r]];
+                    xu[r] = vu[cl[r]];
+                    xe[r] = ld_raw(E + cl[r] * N);
                 }
                 if constexpr (D3 && !IMPL) {
-                    xbd = vbd[cl];
-                    xbu = vbu[cl];
-                    xe2 = ld_raw(E2 + cl * N);
+                    xbd[r] = vbd[cl[r]];
+                    xbu[r] = vbu[cl[r]];
+                    xe2[r] = ld_raw(E2 + cl[r] * N);
                 }
             }
             R vv[N], ww[N];
@@ -616,11 +634,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? (D3 ? 3 : 4) : 2) line4_
                 } else {
                     const R vnx = j + 1 < N ? vv[j + 1] : nv;
                     const R ej = NL ? Ev[j] * hf[j] : Ev[j];
-                    F[j] = lg[j] * (Tnx - Tc[j]) + mu * ej * LM::outer(lim, vv[j], vnx);
+                    F[j] = fma_rn(lg[j], Tnx - Tc[j], mul_rn(mul_rn(mu, ej), LM::outer(lim, vv[j], vnx)));
                 }
                 if constexpr (D3 && !IMPL) {
                     const R wnx = j + 1 < N ? ww[j + 1] : nw;
-                    F[j] += mu2 * (NL ? E2v[j] * hf[j] : E2v[j]) * LM::outer(lim, ww[j], wnx);
+                    F[j] = fma_rn(mul_rn(mu2, NL ? E2v[j] * hf[j] : E2v[j]), LM::outer(lim, ww[j], wnx), F[j]);
                 }
             }
             if (c < m) {
