@@ -134,13 +134,13 @@ struct aniso_ctx {
     bool col_transpose() const { return long_cols() || bc == ANISO_BC_DIRICHLET; }
     bool dirichlet() const { return bc == ANISO_BC_DIRICHLET; }
     int vec() const { return prec == PREC_FP64 ? 2 : 4; }
-    // Grid shapes the vectorised x-then-y path handles: both line lengths a
-    // multiple of the 16-byte vector and short enough for transposed output.
-    // 4: warp-per-line kernel (line4, option value 3); 6: line4 for the lines
-    // it takes and the long-line kernel (line6, 2049-4096 cells, FP32) for
-    // the others, x-then-y steps only; 7: as 6, with lines the cluster kernel
-    // (line7) takes, or the compensated state on line7 in both directions;
-    // 2: line2; 0: none of them.
+    // Grid shapes the vectorised x-then-y path handles: line lengths short
+    // enough for transposed output.  4: warp-per-line kernel (line4, option
+    // value 3; any length, others than multiples of the 16-byte vector in its
+    // ragged form); 6: line4 for the lines it takes and the long-line kernel
+    // (line6, up to 4096 cells in whole vectors) for the others, x-then-y steps
+    // only; 7: as 6, with lines the cluster kernel (line7) takes, or the
+    // compensated state on line7 in both directions; 2: line2; 0: none of them.
     int long_kernel(int n) const
     {
         int a, b, c;
@@ -150,6 +150,22 @@ struct aniso_ctx {
         if (cluster != 0 && line7_config(prec, field_fp16, n, &a, &b, &d)) return 7;
         return 0;
     }
+    // line4 takes lines of n cells: with whole 16-byte vectors, or in its
+    // ragged form (which has no temperature-dependent or 4-step variant).
+    bool line4_whole(int n) const
+    {
+        int a, b, c;
+        size_t d;
+        return line4_config(prec, n, true, l4_warps, seg_chunks, &a, &b, &c, &d);
+    }
+    bool line4_any(int n) const
+    {
+        int a, b, c;
+        size_t d;
+        return line4_whole(n) || (nl_alpha == 0.0 && scheme == ANISO_SCHEME_2STEP &&
+                                  line4_config(prec, n, true, l4_warps, seg_chunks, &a, &b, &c, &d, false, true));
+    }
+    bool whole_vectors() const { return nx % vec() == 0 && ny % vec() == 0; }
     int fast_kind() const
     {
         int a, b, c;
@@ -160,8 +176,7 @@ struct aniso_ctx {
                        ? 7
                        : 0;
         if (fast == 3) {
-            const bool x4 = line4_config(prec, nx, true, l4_warps, seg_chunks, &a, &b, &c, &d);
-            const bool y4 = line4_config(prec, ny, true, l4_warps, seg_chunks, &a, &b, &c, &d);
+            const bool x4 = line4_any(nx), y4 = line4_any(ny);
             if (x4 && y4) return 4;
             const int kx = x4 ? 4 : long_kernel(nx), ky = y4 ? 4 : long_kernel(ny);
             if (kx && ky) return (kx == 7 || ky == 7) ? 7 : 6;
@@ -396,12 +411,13 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     }
     int nthreads;
     size_t smem;
+    const bool ragged = v4 && (n % h->vec() != 0 || n < 2 * h->vec() || !aligned16(in) || !aligned16(out));
     const int seg = v4 && h->seg_chunks == 0 && h->prec == PREC_FP64 ? line4_seg_fp64(n, nlines) : h->seg_chunks;
     const int warps = v4 && transposed && h->l4_warps == 0 && h->seg_chunks == 0 && h->prec == PREC_FP32
                           ? line4_warps_alone(n, nlines)
                           : h->l4_warps;
     bool ok = v4 ? line4_config(h->prec, n, transposed, warps, seg, &J.team, &J.lines_per_block, &nthreads,
-                                &smem)
+                                &smem, false, ragged)
                  : line2_config(h->prec, n, transposed, &J.team, &J.lines_per_block, &nthreads, &smem,
                                 h->seg_chunks);
     if (v4 && ok) J.swz = line4_swizzle(h->prec, n, J.team);
@@ -437,6 +453,7 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     }
     CU(v7   ? launch_line7(h->field_fp16, a, cs, smem, s)
        : v6 ? launch_line6(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s)
+       : ragged ? launch_line4_ragged(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s)
        : v4 ? launch_line4(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s)
             : launch_line2(h->prec, h->field_fp16, a, J.nblocks, nthreads, smem, s, in_lo != nullptr));
     if (h->profile) {
@@ -452,9 +469,15 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
 // transposed y coefficients) and writes T back row-major.
 // With the compensated state the low parts travel the same way (tlo <->
 // tstar_lo), on the cluster kernel.
+static bool fast_alignment(const aniso_ctx *h, const void *T)
+{
+    // (an unaligned T takes line4's ragged form, which only the plain 2-step update has)
+    return aligned16(T) || (h->fast_kind() == 4 && h->nl_alpha == 0.0 && h->scheme == ANISO_SCHEME_2STEP);
+}
+
 static bool use_fast(const aniso_ctx *h, const void *T)
 {
-    return h->fast && !h->dirichlet() && h->order == ANISO_ORDER_XY && h->cyyT && aligned16(T) &&
+    return h->fast && !h->dirichlet() && h->order == ANISO_ORDER_XY && h->cyyT && fast_alignment(h, T) &&
            aligned16(h->tstar) && (!h->kahan || (aligned16(h->tlo) && aligned16(h->tstar_lo))) &&
            h->fast_shape();
 }
@@ -666,8 +689,8 @@ static bool x_first(int order, long long counter)
 // brings the state back to T when it ends in T*.
 static bool fast_any_order(const aniso_ctx *h, const void *T)
 {
-    return h->fast && !h->kahan && !h->dirichlet() && !h->q && h->nl_alpha == 0.0 && h->cyyT && aligned16(T) &&
-           aligned16(h->tstar) && h->fast_kind() == 4;
+    return h->fast && !h->kahan && !h->dirichlet() && !h->q && h->nl_alpha == 0.0 && h->cyyT &&
+           fast_alignment(h, T) && aligned16(h->tstar) && h->fast_kind() == 4;
 }
 
 static int enqueue_steps_any_order(aniso_ctx *h, void *T, double dt, int nsteps, long long counter0,
@@ -1120,6 +1143,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         long long table = -1;  // line4: offset of the block -> job table, or -1
         int diag_region = -1;  // line4 y-update with diagnostics: its partials region
         int tmem = 0;          // line4: gamma in tensor memory
+        int ragged = 0;        // line4: the form for any length and alignment
         int step = 0;          // the call's step the launch belongs to
     };
     std::vector<unsigned char> blob;
@@ -1211,19 +1235,25 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         // one block size for the launch: the largest any job needs, then every
         // job's lines per block for that many warps
         int nthreads = 0;
+        const int vec = prec == PREC_FP64 ? 2 : 4;
+        auto ragged = [&](const Line2Job &J) {
+            return J.n % vec != 0 || J.n < 2 * vec || !aligned16(J.Tin) || !aligned16(J.Tout);
+        };
         for (auto &J : jobs) {
             int nt;
             size_t sm;
-            if (line4_config(prec, J.n, true, warps, seg, &J.team, &J.lines_per_block, &nt, &sm))
+            if (line4_config(prec, J.n, true, warps, seg, &J.team, &J.lines_per_block, &nt, &sm, false, ragged(J)))
                 nthreads = std::max(nthreads, nt);
         }
         // Per job: its resident blocks per SM in the shared-memory form and, when
         // the lines fit it, in the tensor-memory form (whose TMEM columns also
         // cap the blocks an SM holds); the form with more blocks wins.
+        // (Lines that are no whole vectors, or whose arrays are not aligned to
+        // them, run in the kernel's ragged form: classes of their own.)
         struct Cls {
             int occ;
             size_t sm;
-            bool tm;
+            int form;  // 0 shared memory, 1 tensor memory, 2 ragged
         };
         const bool tm_on = b->hs[0]->tmem != 0 && prec == PREC_FP32;
         std::vector<Cls> cls(jobs.size());
@@ -1231,27 +1261,28 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             Line2Job &J = jobs[k];
             int nt = 0;
             size_t sm = 0;
-            if (!line4_config(prec, J.n, true, nthreads / 32, seg, &J.team, &J.lines_per_block, &nt, &sm) ||
+            if (!line4_config(prec, J.n, true, nthreads / 32, seg, &J.team, &J.lines_per_block, &nt, &sm, false,
+                              ragged(J)) ||
                 nt != nthreads)
                 shape_rc = fail(ANISO_ERR_UNSUPPORTED, "batch: line length %d does not fit the block shape", J.n);
             J.swz = line4_swizzle(prec, J.n, J.team);
             int occ = line4_blocks_per_sm(prec, fp16, b->hs[0]->limiter, nthreads, sm, false);
-            cls[k] = {occ > 0 ? occ : 0, sm, false};
+            cls[k] = {occ > 0 ? occ : 0, sm, ragged(J) ? 2 : 0};
             int t0, t1, t2;
             size_t smt = 0;
-            if (tm_on && line4_config(prec, J.n, true, nthreads / 32, seg, &t0, &t1, &t2, &smt, true)) {
+            if (tm_on && !ragged(J) && line4_config(prec, J.n, true, nthreads / 32, seg, &t0, &t1, &t2, &smt, true)) {
                 const int occt = line4_blocks_per_sm(prec, fp16, b->hs[0]->limiter, nthreads, smt, true,
                                                      line4_tm_cols(J.n, J.team));
-                if (occt > cls[k].occ) cls[k] = {occt, smt, true};
+                if (occt > cls[k].occ) cls[k] = {occt, smt, 1};
             }
         }
         // per form, classes in ascending occupancy (largest lines first); at
         // most three a form, the highest-occupancy ones merged
         int region = 0;
-        for (int form = 1; form >= 0; --form) {
+        for (int form : {1, 0, 2}) {
             std::vector<int> occs;
             for (auto &c : cls)
-                if (c.tm == (form == 1)) occs.push_back(c.occ);
+                if (c.form == form) occs.push_back(c.occ);
             std::sort(occs.begin(), occs.end());
             occs.erase(std::unique(occs.begin(), occs.end()), occs.end());
             // (merging never drops the lowest class: its range reaches up to the next kept one)
@@ -1262,7 +1293,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                 size_t smem = 0;
                 int blocks = 0;
                 for (size_t k = 0; k < jobs.size(); ++k) {
-                    if (cls[k].tm != (form == 1) || cls[k].occ < lo || cls[k].occ >= hi) continue;
+                    if (cls[k].form != form || cls[k].occ < lo || cls[k].occ >= hi) continue;
                     Line2Job J = jobs[k];
                     smem = std::max(smem, cls[k].sm);
                     J.block0 = blocks;
@@ -1273,7 +1304,8 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                 if (part.empty()) continue;
                 Launch L{kind_xy == 0 ? 7 : 8, blob.size(), (int)part.size(), blocks, nthreads, smem};
                 L.group = group;
-                L.tmem = form;
+                L.tmem = form == 1;
+                L.ragged = form == 2;
                 if (kind_xy == 1 && diag) L.diag_region = region;
                 ++region;
                 const unsigned char *p = reinterpret_cast<const unsigned char *>(part.data());
@@ -1423,11 +1455,14 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                     J.per_line = per;
                     J.per_cross = per;
                     J.transpose_out = 1;
-                    J.diag_slot = (diag && phase == 1) ? k * max_steps + s : -1;
+                    // (recorded for grids of whole, aligned vectors: the ragged form's extra elements are not cells)
+                    J.diag_slot =
+                        (diag && phase == 1 && h->whole_vectors() && aligned16(T[k])) ? k * max_steps + s : -1;
                     int t5, l5, n5;
                     size_t s5;
                     const int fk = h->fast_kind();
-                    if ((fk == 4 || fk == 6) && tma_mode && !(diag && phase == 1) && line5_available() &&
+                    if ((fk == 4 || fk == 6) && tma_mode && J.nlines % 4 == 0 && aligned16(J.Tin) &&
+                        aligned16(J.Tout) && !(diag && phase == 1) && line5_available() &&
                         line5_config(prec, fp16, J.n, &t5, &l5, &n5, &s5)) {
                         Line5Job J5{};
                         J5.Tout = J.Tout;
@@ -1444,8 +1479,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                             continue;
                         }
                     }
-                    if (fk == 6 && !line4_config(prec, J.n, true, b->hs[0]->l4_warps, b->hs[0]->seg_chunks, &nt,
-                                                 &nt, &nt, &sm)) {
+                    if (fk == 6 && !h->line4_any(J.n)) {
                         // above line4's limit: the long-line kernel
                         line6_config(prec, fp16, J.n, &J.team, &J.lines_per_block, &nt, &sm,
                                      b->hs[0]->l4_warps == 8 ? 2 : 4);
@@ -1611,15 +1645,19 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             if (L.table >= 0)
                 a.block_job = reinterpret_cast<const int *>(static_cast<unsigned char *>(b->d_jobs) + L.table);
             a.tmem = L.tmem;
+            auto launch4 = [&](const Line2Args &args) {
+                return L.ragged ? launch_line4_ragged(prec, fp16, args, L.nblocks, L.nthreads, L.smem, st)
+                                : launch_line4(prec, fp16, args, L.nblocks, L.nthreads, L.smem, st);
+            };
             if (L.diag_region >= 0) {
                 a.diag_part = b->d_part + (size_t)L.diag_region * part_blocks;
-                cudaError_t e = launch_line4(prec, fp16, a, L.nblocks, L.nthreads, L.smem, st);
+                cudaError_t e = launch4(a);
                 if (e != cudaSuccess) return e;
                 return launch_diag_finish(a.jobs, L.njobs, a.diag_part, b->d_ring, st);
             }
             a.limiter = b->hs[0]->limiter;
             a.err = err;
-            return launch_line4(prec, fp16, a, L.nblocks, L.nthreads, L.smem, st);
+            return launch4(a);
         } else if (L.kind >= 2) {
             Line2Args a{};
             a.jobs = reinterpret_cast<const Line2Job *>(static_cast<unsigned char *>(b->d_jobs) + L.offset);

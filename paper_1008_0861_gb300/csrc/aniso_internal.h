@@ -174,9 +174,13 @@ cudaError_t launch_source(int prec, void *T, const void *Q, double dt, size_t n,
 // chunks per lane (0 = default of 4), which sets the team size and so the
 // PCR depth.
 // tmem: the tensor-memory form (FP32, four-warp blocks, at most 8 chunks a
-// lane); false when the line does not fit it.
+// lane); false when the line does not fit it.  ragged: the form for lines that
+// are no multiple of the 16-byte vector, or arrays that are not aligned to it
+// (2-D updates with the transverse term and constant diffusivity).
 bool line4_config(int prec, int n, bool transposed, int warps, int seg_chunks, int *team, int *lines_per_block,
-                  int *nthreads, size_t *smem, bool tmem = false);
+                  int *nthreads, size_t *smem, bool tmem = false, bool ragged = false);
+cudaError_t launch_line4_ragged(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
+                                cudaStream_t s);
 cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads,
                          size_t smem, cudaStream_t s);
 // Long lines (line6): FP32 2048 < n <= 4096, FP64 1024 < n <= 4096, teams of

@@ -96,7 +96,7 @@ int line4_tm_cols(int n, int team)
 // from 256 cells a line on both rules agree.
 int line4_seg_fp64(int n, int nlines)
 {
-    const int m = n / 2;
+    const int m = (n + 1) / 2;
     int P = 1, top = 1, best = 4;
     while (P * 2 <= m / 4 && P < 32) P *= 2;
     while (top * 2 <= m && top < 32) top *= 2;
@@ -124,7 +124,7 @@ int line4_warps_alone(int n, int nlines)
 {
     int team, lpb, nt;
     size_t smem;
-    if (!line4_config(PREC_FP32, n, true, 8, 0, &team, &lpb, &nt, &smem) || lpb != 8 || nt != 256) return 0;
+    if (!line4_config(PREC_FP32, (n + 3) & ~3, true, 8, 0, &team, &lpb, &nt, &smem) || lpb != 8 || nt != 256) return 0;
     const long blocks = ((long)nlines + 7) / 8, resident = (long)((SMEM_LIMIT - 1024) / (smem + 1024));
     return blocks >= 96 && blocks <= 152 * (resident < 4 ? resident : 4) ? 8 : 0;
 }
@@ -142,7 +142,7 @@ int line4_warps_alone(int n, int nlines)
 int line4_swizzle(int prec, int n, int team)
 {
     const int N = prec == PREC_FP64 ? 2 : 4;
-    const int m = n / N, P = team;
+    const int m = (n + N - 1) / N, P = team;
     if (P < 8 || m < 8) return 0;  // a quarter warp spans several lines
     const int U = m / P, rr = m % P, V = U + (rr ? 1 : 0);
     const int mfull = m & ~7;

@@ -60,6 +60,38 @@ __device__ __forceinline__ void unpack_raw(const uint2 &v, float *o)
     o[3] = b.y;
 }
 
+// The same 16 bytes of T / N coefficients element by element, from any
+// address: elements a, b, c, d of a row.  T goes by plain loads (a chained
+// launch starts while its input is still written), coefficients by read-only
+// ones.
+template <bool RO, typename E> __device__ __forceinline__ E ld1(const E *p)
+{
+    if constexpr (RO) return __ldg(p);
+    else return *p;
+}
+template <bool RO> __device__ __forceinline__ float4 ld_elem(const float *r, int a, int b, int c, int d)
+{
+    return make_float4(ld1<RO>(r + a), ld1<RO>(r + b), ld1<RO>(r + c), ld1<RO>(r + d));
+}
+template <bool RO> __device__ __forceinline__ uint2 ld_elem(const __half *r, int a, int b, int c, int d)
+{
+    const unsigned short *u = reinterpret_cast<const unsigned short *>(r);
+    const unsigned x = ld1<RO>(u + a), y = ld1<RO>(u + b), z = ld1<RO>(u + c), w = ld1<RO>(u + d);
+    return make_uint2(x | (y << 16), z | (w << 16));
+}
+template <bool RO> __device__ __forceinline__ double2 ld_elem(const double *r, int a, int b, int, int)
+{
+    return make_double2(ld1<RO>(r + a), ld1<RO>(r + b));
+}
+// Chunk c of a row of n cells; elements from n on are taken at p1.
+template <int N, bool RO, typename E> __device__ __forceinline__ auto ld_ragged(const E *row, int c, int n, int p1)
+{
+    const int p = c * N;
+    if (p + N <= n) return ld_elem<RO>(row + p, 0, 1, 2, 3);
+    auto at = [n, p1](int k) { return k < n ? k : p1; };
+    return ld_elem<RO>(row, at(p), at(p + 1), at(p + 2), at(p + 3));
+}
+
 // Bulk prefetch of a byte range into L2 (no destination, no completion).
 __device__ __forceinline__ void l2_prefetch(const void *p, size_t bytes)
 {
@@ -384,6 +416,13 @@ __device__ __forceinline__ void tm_ld4(unsigned taddr, float *o)
 }
 __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// RAG: lines of any length and arrays of any alignment.  The line's last
+// chunk holds its last nv = 1 .. N cells; loads and line-major stores go element
+// by element (the four elements of a chunk share their sectors, so the extra
+// instructions are most of the cost); an element past the line reads the cell
+// after it (the wrap or the mirrored ghost), which the last face needs.  The
+// last segment ends at position nv - 1 of its last chunk.  A line's solve is
+// the same as with whole chunks.
 // IMPL: a purely implicit update (no transverse term, mu = mu2 = 0: the second
 // half-update of each axis in the 4-step scheme); neighbouring lines and
 // transverse coefficients are then neither loaded nor limited.
@@ -393,10 +432,11 @@ __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sy
 // lane's chunks of T_old wait there too, from the flux phase to phase C
 // (4 V + 4 V columns of the block's 32 or 64).
 template <typename R, typename C, bool VL, bool D3 = false, bool NL = false, bool IMPL = false, bool TM = false,
-          int RING = 1>
+          int RING = 1, bool RAG = false>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4) : 2) line4_kernel(Line2Args args)
 {
     static_assert(!TM || (sizeof(R) == 4 && !D3), "TMEM line state: FP32 2-D only");
+    static_assert(!RAG || (!D3 && !NL && !IMPL && !TM), "ragged lines: the plain 2-D update only");
     typedef typename V16<R>::T VT;
     constexpr int N = V16<R>::N;
     constexpr int LOGN = N == 4 ? 2 : 1;
@@ -416,7 +456,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     __syncthreads();
 
     const int lim = args.limiter;
-    const int P = J.team, n = J.n, m = n / N, nl = J.nlines, LPB = J.lines_per_block;
+    const int P = J.team, n = J.n, m = RAG ? (n + N - 1) / N : n / N, nl = J.nlines, LPB = J.lines_per_block;
+    const int nv = RAG ? n - (m - 1) * N : N;  // cells of the last chunk
     const int logP = __ffs(P) - 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int logL = 5 - logP;  // 32 / P lines per warp
@@ -508,18 +549,27 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         R wcar = R(0);               // the same for the second transverse axis (D3)
         // the loads of the next RING rounds are issued before a round's arithmetic
         typedef decltype(ld_raw(G)) CT;
+        const int p1 = J.per_line ? 0 : n - 1;
+        auto ldT = [&](const VT *v, const R *row, int c) -> VT {
+            if constexpr (RAG) return ld_ragged<N, false>(row, c, n, p1);
+            else return v[c];
+        };
+        auto ldC = [&](const C *row, int c) -> CT {
+            if constexpr (RAG) return ld_ragged<N, true>(row, c, n, p1);
+            else return ld_raw(row + c * N);
+        };
         int cl[RING];
         VT xc[RING], xd[RING], xu[RING], xbd[RING], xbu[RING];
         CT xg[RING], xe[RING], xe2[RING];
 #pragma unroll
         for (int r = 0; r < RING; ++r) {
             cl[r] = min((max(V - 1 - r, 0) << logP) + t, m - 1);
-            xc[r] = xd[r] = xu[r] = xbd[r] = xbu[r] = vc[cl[r]];
-            xg[r] = xe[r] = xe2[r] = ld_raw(G + cl[r] * N);
+            xc[r] = xd[r] = xu[r] = xbd[r] = xbu[r] = ldT(vc, rc, cl[r]);
+            xg[r] = xe[r] = xe2[r] = ldC(G, cl[r]);
             if constexpr (!IMPL) {
-                xd[r] = vd[cl[r]];
-                xu[r] = vu[cl[r]];
-                xe[r] = ld_raw(E + cl[r] * N);
+                xd[r] = ldT(vd, rd, cl[r]);
+                xu[r] = ldT(vu, ru, cl[r]);
+                xe[r] = ldC(E, cl[r]);
             }
             if constexpr (D3 && !IMPL) {
                 xbd[r] = vbd[cl[r]];
@@ -532,7 +582,6 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         // 3-D and temperature-dependent forms, short of registers, load it
         // where it is used)
         constexpr bool EARLY = !D3 && !NL;
-        const int p1 = J.per_line ? 0 : n - 1;
         R eT = R(0), eU = R(0), eD = R(0);
         if constexpr (EARLY) {
             eT = rc[p1];
@@ -572,12 +621,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
             const int cur = cl[r];
             if (v >= RING) {
                 cl[r] = ((v - RING) << logP) + t;  // always < m
-                xc[r] = vc[cl[r]];
-                xg[r] = ld_raw(G + cl[r] * N);
+                xc[r] = ldT(vc, rc, cl[r]);
+                xg[r] = ldC(G, cl[r]);
                 if constexpr (!IMPL) {
-                    xd[r] = vd[cl[r]];
-                    xu[r] = vu[cl[r]];
-                    xe[r] = ld_raw(E + cl[r] * N);
+                    xd[r] = ldT(vd, rd, cl[r]);
+                    xu[r] = ldT(vu, ru, cl[r]);
+                    xe[r] = ldC(E, cl[r]);
                 }
                 if constexpr (D3 && !IMPL) {
                     xbd[r] = vbd[cl[r]];
@@ -655,6 +704,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     {
         R Fpend = R(0), lgpend = R(0), Flast = R(0);
         R ro[N], ao[N], go[N];  // maps of the chunk above, waiting for its row 0
+        bool pend = false;      // RAG: the segment ends in row 0 of its last chunk, whose lower face is still to come
 #pragma unroll
         for (int v = 0; v < N; ++v) ro[v] = ao[v] = go[v] = R(0);
         // (TMEM form: every lane runs all V rounds, so that the warp-wide TMEM
@@ -669,7 +719,25 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
             R F[N], lg[N], co[N], cao[N], cgo[N];
             V16<R>::unpack(sA[swz(c)], F);
             V16<R>::unpack(sB[swz(c)], lg);
-            if (u == Ut - 1) {
+            if (RAG && u == Ut - 1 && c == m - 1 && nv < N) {
+                // the line's last cell is position nv - 1
+                Flast = F[0];
+                lge = lg[0];
+                pend = nv == 1;
+#pragma unroll
+                for (int j = 1; j < N; ++j) {
+                    co[j] = cao[j] = cgo[j] = R(0);
+                    if (j == nv - 1) {
+                        Flast = F[j];
+                        lge = lg[j];
+                        lgem = lg[j - 1];
+                        re = F[j] - F[j - 1];
+                    }
+                }
+#pragma unroll
+                for (int j = N - 2; j >= 1; --j)
+                    if (j < nv - 1) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
+            } else if (u == Ut - 1) {
                 // row e (last cell of the segment) enters the reduced system
                 lge = lg[N - 1];
                 lgem = lg[N - 2];
@@ -680,7 +748,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
                 for (int j = N - 2; j >= 1; --j) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             } else {
                 // row 0 of the chunk above, then this chunk's rows N-1 .. 1
-                sg.elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
+                if (RAG && pend) {
+                    lgem = lg[N - 1];
+                    re = Flast - F[N - 1];
+                    pend = false;
+                } else {
+                    sg.elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
+                }
                 sA[swz(c + 1)] = V16<R>::pack(ro);
                 sB[swz(c + 1)] = V16<R>::pack(ao);
                 if constexpr (TM) {
@@ -709,7 +783,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         const int tp = (t - 1) & (P - 1);
         const R Fprev = __shfl_sync(full, Flast, tp, P), lgprev = __shfl_sync(full, lge, tp, P);
         lgs = lgprev;
-        sg.elim(Fpend, Fprev, lgpend, lgprev, ro[0], ao[0], go[0]);
+        if (RAG && pend) {  // a segment of one cell: its row is row e
+            lgem = lgprev;
+            re = Flast - Fprev;
+        } else {
+            sg.elim(Fpend, Fprev, lgpend, lgprev, ro[0], ao[0], go[0]);
+        }
         sA[swz(c_lo)] = V16<R>::pack(ro);
         sB[swz(c_lo)] = V16<R>::pack(ao);
         if constexpr (TM) {
@@ -725,9 +804,13 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     // (TMEM form: T_old is in tensor memory already)
     const VT *vcC = reinterpret_cast<const VT *>(rc);
     VT pre0{}, pre1{};
+    auto ld_old = [&](int c) -> VT {
+        if constexpr (RAG) return ld_ragged<N, false>(rc, c, n, n - 1);
+        else return vcC[c];
+    };
     if constexpr (!TM) {
-        pre0 = pre1 = vcC[t];  // t < P <= m
-        if (t + P < m) pre1 = vcC[t + P];
+        pre0 = pre1 = ld_old(t);  // t < P <= m
+        if (t + P < m) pre1 = ld_old(t + P);
     }
 
     // ---- R: reduced system of the line in the segment-end unknowns
@@ -755,6 +838,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 d[j] = (u == Ut - 1 && j == N - 1) ? X : r4[j] - a4[j] * dprev - g4[j] * X;
+                if (RAG && c == m - 1 && j >= nv - 1) d[j] = j == nv - 1 ? X : R(0);
                 dprev = d[j];
             }
             sA[swz(c)] = V16<R>::pack(d);
@@ -779,7 +863,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
                 if (c >= m) break;
                 V16<R>::unpack(pre0, to);
                 pre0 = pre1;  // two chunks in flight
-                if (c + 2 * P < m) pre1 = vcC[c + 2 * P];
+                if (c + 2 * P < m) pre1 = ld_old(c + 2 * P);
             }
             V16<R>::unpack(sA[swz(c)], d);
             R sum = R(0);
@@ -802,7 +886,14 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
                 }
             }
             if (!J.transpose_out) {
-                if (active) vout[c] = V16<R>::pack(to);
+                if constexpr (RAG) {
+                    R *o = static_cast<R *>(J.Tout) + (size_t)lc * n + (size_t)c * N;
+#pragma unroll
+                    for (int j = 0; j < N; ++j)
+                        if (active && c * N + j < n) o[j] = to[j];
+                } else {
+                    if (active) vout[c] = V16<R>::pack(to);
+                }
             } else {
                 sA[swz(c)] = V16<R>::pack(to);
             }
@@ -817,7 +908,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         __syncthreads();
         R *out = static_cast<R *>(J.Tout);
         const int groups = LPB >> LOGN, logG = __ffs(groups) - 1;
-        const bool vec_ok = (nl & (N - 1)) == 0;
+        const bool vec_ok = (nl & (N - 1)) == 0 && (!RAG || (reinterpret_cast<uintptr_t>(out) & 15) == 0);
         const int pairs = groups == 1 ? n : (((n + 15) & ~15) << logG);
         for (int idx = threadIdx.x; idx < pairs; idx += blockDim.x) {
             const int p = groups == 1 ? idx : (((idx >> (4 + logG)) << 4) | (idx & 15));

@@ -132,14 +132,14 @@ bool line2_config(int prec, int n, bool transposed, int *team, int *lines_per_bl
 // seg_chunks (default 4: 16 FP32 / 8 FP64 cells) chunks per lane or more, at
 // most 16 chunks a lane; the warp's shared area holds 3 arrays of its lines' chunks.  Blocks
 // of `warps` warps (default 4); with a transposed output the block's line
-// count must fill whole 16-byte stores.
+// count must fill whole 16-byte stores.  ragged: the form for any length.
 bool line4_config(int prec, int n, bool transposed, int warps, int seg_chunks, int *team, int *lines_per_block,
-                  int *nthreads, size_t *smem, bool tmem)
+                  int *nthreads, size_t *smem, bool tmem, bool ragged)
 {
     const int N = prec == PREC_FP64 ? 2 : 4;
-    if (n % N != 0 || n < 2 * N) return false;
+    if (ragged ? tmem || n < 3 : n % N != 0 || n < 2 * N) return false;
     if (transposed && n > MAX_LINE2_TRANSPOSED) return false;
-    const int m = n / N, sc = seg_chunks > 0 ? seg_chunks : 4;
+    const int m = (n + N - 1) / N, sc = seg_chunks > 0 ? seg_chunks : 4;
     int P = pow2floor(m / sc > 0 ? m / sc : 1);
     if (P > 32) P = 32;
     const int U = m / P, V = U + (m % P ? 1 : 0);
