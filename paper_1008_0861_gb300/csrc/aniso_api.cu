@@ -1645,6 +1645,8 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             if (L.table >= 0)
                 a.block_job = reinterpret_cast<const int *>(static_cast<unsigned char *>(b->d_jobs) + L.table);
             a.tmem = L.tmem;
+            a.limiter = b->hs[0]->limiter;
+            a.err = err;
             auto launch4 = [&](const Line2Args &args) {
                 return L.ragged ? launch_line4_ragged(prec, fp16, args, L.nblocks, L.nthreads, L.smem, st)
                                 : launch_line4(prec, fp16, args, L.nblocks, L.nthreads, L.smem, st);
@@ -1655,8 +1657,6 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                 if (e != cudaSuccess) return e;
                 return launch_diag_finish(a.jobs, L.njobs, a.diag_part, b->d_ring, st);
             }
-            a.limiter = b->hs[0]->limiter;
-            a.err = err;
             return launch4(a);
         } else if (L.kind >= 2) {
             Line2Args a{};

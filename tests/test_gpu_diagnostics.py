@@ -120,3 +120,29 @@ def test_diagnostics_are_nan_where_the_y_update_is_not_the_warp_per_line_kernel(
         lib.aniso_batch_destroy(b)
         for g in grids:
             g.close()
+
+
+def test_diagnostics_keep_the_limiter_and_the_error_flag(lib):
+    """A recorded call runs the batch's limiter, and reports a non-finite
+    temperature, like an unrecorded one."""
+    import torch
+    inst = W.random_instance(128, 96, seed=3, dt_factor=50.0, nsteps=2)
+    a, c = (GpuGrid(lib, inst, 1, limiter=2) for _ in range(2))
+    lib.aniso_set_option(a.h, lib.ANISO_OPT_DIAGNOSTICS, 1)
+    try:
+        ba, bc = lib.aniso_batch_create([a.h]), lib.aniso_batch_create([c.h])
+        for b, g in ((ba, a), (bc, c)):
+            lib.aniso_step_batched(b, [g.T], [inst.dt], [2])
+        torch.cuda.synchronize()
+        assert torch.equal(a.T, c.T)
+        lib.aniso_sync(a.h)
+        a.T[5, 7] = float("nan")
+        lib.aniso_step_batched(ba, [a.T], [inst.dt], [2])
+        with pytest.raises(lib.AnisoError) as ei:
+            lib.aniso_sync(a.h)
+        assert ei.value.code == lib.ANISO_ERR_NONFINITE
+        lib.aniso_batch_destroy(ba)
+        lib.aniso_batch_destroy(bc)
+    finally:
+        a.close()
+        c.close()
