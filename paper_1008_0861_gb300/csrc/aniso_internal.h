@@ -133,7 +133,7 @@ struct Line2Args {
     // memory (the launch's shared memory then holds two arrays, not three)
     int tmem;
     // 1: launched to start while the kernel before it in the stream drains
-    // (programmatic dependent launch); never the first launch of a captured call
+    // (programmatic dependent launch); in a capture never a call's first launch
     int chained;
 };
 // Finish the diagnostics of one line4 launch: for every job, the partials of
@@ -206,6 +206,8 @@ int line4_blocks_per_sm(int prec, int coef_fp16, int limiter, int nthreads, size
 int line4_seg_fp64(int n, int nlines);
 // warps a block (0: the default) for an FP32 update of nlines lines of n cells launched alone.
 int line4_warps_alone(int n, int nlines);
+// dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each.
+size_t line4_smem_alone(int nblocks, size_t smem);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.
 int line4_tm_cols(int n, int team);
 // Chunks of padding after each warp's shared area in the FP32 line4 kernel
@@ -249,7 +251,10 @@ cudaError_t launch_line2(int prec, int coef_fp16, const Line2Args &a, int nblock
 // the transposed copies cyyT/cyxT [nx][ny] are each optional (null).
 cudaError_t launch_face_coeffs(int bprec, int coef, const void *bx, const void *by, int nx, int ny,
                                int bc, double kappa, void *cxx, void *cxy, void *cyy, void *cyx,
-                               void *cyyT, void *cyxT, cudaStream_t s);
+                               void *cyyT, void *cyxT, cudaStream_t s, bool chained = false);
+// Whether a call's first kernel may be launched chained: not into a capture,
+// where what comes before it may be no kernel.
+bool may_chain(cudaStream_t s);
 // out[c][r] = in[r][c] for an rows x cols array of 4- or 8-byte elements.
 cudaError_t launch_transpose(int elem_bytes, const void *in, void *out, int rows, int cols,
                              cudaStream_t s);

@@ -129,6 +129,23 @@ int line4_warps_alone(int n, int nlines)
     return blocks >= 96 && blocks <= 152 * (resident < 4 ? resident : 4) ? 8 : 0;
 }
 
+// Dynamic shared memory for a chained FP32 launch of a grid alone: enough that
+// an SM holds no more than its share of the blocks.  A chained launch's blocks
+// are placed while their predecessor drains, on whichever SMs are free first, and
+// with room for more one SM got two or three of them and another none.  us with
+// the natural size / this one: 1024^2 9.69 / 9.03 an update, 1152^2 11.5 / 10.9;
+// field and step at 1024^2 45.5 / 36.9.  Short lines (under 40 KB a block) keep
+// theirs: there the SMs' switch to another split of L1 and shared memory costs
+// more (512^2, field and step 19.5 / 24.9), as does the L1 that the ragged
+// form's loads live on (1001^2 13.6 / 14.2).
+size_t line4_smem_alone(int nblocks, size_t smem)
+{
+    const int share = (nblocks + 151) / 152;
+    if (share > 4 || smem < 40 * 1024) return smem;
+    const size_t least = (size_t)228 * 1024 / (share + 1) - 1024 + 16;
+    return smem > least ? smem : least;
+}
+
 // The kernel keeps 16-byte chunk c of a line at c ^ ((c >> s) & 7) inside
 // its group of 8 chunks (the last, incomplete group unswizzled).  The
 // coalesced phases have the 8 lanes of a quarter warp touch one whole group,

@@ -61,35 +61,25 @@ __device__ __forceinline__ void unpack_raw(const uint2 &v, float *o)
 }
 
 // The same 16 bytes of T / N coefficients element by element, from any
-// address: elements a, b, c, d of a row.  T goes by plain loads (a chained
-// launch starts while its input is still written), coefficients by read-only
-// ones.
-template <bool RO, typename E> __device__ __forceinline__ E ld1(const E *p)
+// address: elements a, b, c, d of a row.
+__device__ __forceinline__ float4 ld_elem(const float *r, int a, int b, int c, int d)
 {
-    if constexpr (RO) return __ldg(p);
-    else return *p;
+    return make_float4(r[a], r[b], r[c], r[d]);
 }
-template <bool RO> __device__ __forceinline__ float4 ld_elem(const float *r, int a, int b, int c, int d)
-{
-    return make_float4(ld1<RO>(r + a), ld1<RO>(r + b), ld1<RO>(r + c), ld1<RO>(r + d));
-}
-template <bool RO> __device__ __forceinline__ uint2 ld_elem(const __half *r, int a, int b, int c, int d)
+__device__ __forceinline__ uint2 ld_elem(const __half *r, int a, int b, int c, int d)
 {
     const unsigned short *u = reinterpret_cast<const unsigned short *>(r);
-    const unsigned x = ld1<RO>(u + a), y = ld1<RO>(u + b), z = ld1<RO>(u + c), w = ld1<RO>(u + d);
+    const unsigned x = u[a], y = u[b], z = u[c], w = u[d];
     return make_uint2(x | (y << 16), z | (w << 16));
 }
-template <bool RO> __device__ __forceinline__ double2 ld_elem(const double *r, int a, int b, int, int)
-{
-    return make_double2(ld1<RO>(r + a), ld1<RO>(r + b));
-}
+__device__ __forceinline__ double2 ld_elem(const double *r, int a, int b, int, int) { return make_double2(r[a], r[b]); }
 // Chunk c of a row of n cells; elements from n on are taken at p1.
-template <int N, bool RO, typename E> __device__ __forceinline__ auto ld_ragged(const E *row, int c, int n, int p1)
+template <int N, typename E> __device__ __forceinline__ auto ld_ragged(const E *row, int c, int n, int p1)
 {
     const int p = c * N;
-    if (p + N <= n) return ld_elem<RO>(row + p, 0, 1, 2, 3);
+    if (p + N <= n) return ld_elem(row + p, 0, 1, 2, 3);
     auto at = [n, p1](int k) { return k < n ? k : p1; };
-    return ld_elem<RO>(row, at(p), at(p + 1), at(p + 2), at(p + 3));
+    return ld_elem(row, at(p), at(p + 1), at(p + 2), at(p + 3));
 }
 
 // Bulk prefetch of a byte range into L2 (no destination, no completion).
@@ -99,42 +89,12 @@ __device__ __forceinline__ void l2_prefetch(const void *p, size_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"((unsigned)bytes) : "memory");
 }
 
-// Programmatic dependent launch: a kernel launched with args.chained may start
-// while the one before it in the stream still runs.  It waits here, before it
-// first touches memory the other writes, and then lets the next one start.
-// (Both are no-ops in a plain launch.)
-__device__ __forceinline__ void chain_wait()
-{
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
 // Host: a launch of kern(a) in a.chained mode or plainly.
 template <typename K>
 static cudaError_t launch_line_kernel(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s,
                                       int cluster = 0)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)nblocks, 1, 1);
-    cfg.blockDim = dim3((unsigned)nthreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[2];
-    unsigned n = 0;
-    if (cluster > 0) {
-        at[n].id = cudaLaunchAttributeClusterDimension;
-        at[n].val.clusterDim.x = (unsigned)cluster;
-        at[n].val.clusterDim.y = 1;
-        at[n].val.clusterDim.z = 1;
-        ++n;
-    }
-    if (a.chained) {
-        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        at[n].val.programmaticStreamSerializationAllowed = 1;
-        ++n;
-    }
-    cfg.attrs = at;
-    cfg.numAttrs = n;
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    return launch_kernel(kern, dim3((unsigned)nblocks), dim3((unsigned)nthreads), smem, s, a.chained != 0, cluster, a);
 }
 
 __device__ __forceinline__ float frcp_approx(float x)
@@ -492,6 +452,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     // (what came before is the kernel's own arguments and indices; batched
     // launches, the only ones in the tensor-memory form, are never chained)
     if (!TM && !args.jobs) chain_wait();
+    if constexpr (!TM) {  // (the kernel before may have written the coefficients)
+        after_wait(G);
+        after_wait(E);
+        if constexpr (D3) after_wait(E2);
+    }
 
     // The block's input rows (its lines and the two neighbouring lines of T,
     // its coefficient rows) start streaming into L2 at once, so that the
@@ -551,11 +516,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         typedef decltype(ld_raw(G)) CT;
         const int p1 = J.per_line ? 0 : n - 1;
         auto ldT = [&](const VT *v, const R *row, int c) -> VT {
-            if constexpr (RAG) return ld_ragged<N, false>(row, c, n, p1);
+            if constexpr (RAG) return ld_ragged<N>(row, c, n, p1);
             else return v[c];
         };
         auto ldC = [&](const C *row, int c) -> CT {
-            if constexpr (RAG) return ld_ragged<N, true>(row, c, n, p1);
+            if constexpr (RAG) return ld_ragged<N>(row, c, n, p1);
             else return ld_raw(row + c * N);
         };
         int cl[RING];
@@ -805,7 +770,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     const VT *vcC = reinterpret_cast<const VT *>(rc);
     VT pre0{}, pre1{};
     auto ld_old = [&](int c) -> VT {
-        if constexpr (RAG) return ld_ragged<N, false>(rc, c, n, n - 1);
+        if constexpr (RAG) return ld_ragged<N>(rc, c, n, n - 1);
         else return vcC[c];
     };
     if constexpr (!TM) {

@@ -95,6 +95,8 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
     const unsigned full = 0xffffffffu;
 
     chain_wait();
+    after_wait(G);
+    after_wait(E);
     if (threadIdx.x == 0) {  // the block's rows into L2 (a hint)
         const int f0 = line0 > 0 ? line0 - 1 : line0, f1 = min(line0 + LPB + 1, nl), g1 = min(line0 + LPB, nl);
         l2_prefetch(Tin + (size_t)f0 * n, (size_t)(f1 - f0) * n * sizeof(R));

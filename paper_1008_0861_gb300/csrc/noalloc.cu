@@ -127,6 +127,7 @@ bool line_launch(int prec, int n, int nlines, const void *in, void *out, const v
     J.transpose_out = 1;
     J.swz = line4_swizzle(prec, n, J.team);
     J.nblocks = (nlines + J.lines_per_block - 1) / J.lines_per_block;
+    if (prec == PREC_FP32 && !L->ragged) L->smem = line4_smem_alone(J.nblocks, L->smem);
     return true;
 }
 
@@ -181,9 +182,9 @@ extern "C" int aniso_step_noalloc(int nx, int ny, double dx, double dy, double c
     LineLaunch lx, ly;
     if (line_launch(precision, nx, ny, T, tstar, cxx, cxy, lamx, mu, per, err, &lx) &&
         line_launch(precision, ny, nx, tstar, T, cyy, cyx, lamy, mu, per, err, &ly)) {
-        e = launch_face_coeffs(precision, coef, bx, by, nx, ny, bc, kappa, cxx, cxy, nullptr, nullptr, cyy, cyx, s);
+        e = launch_face_coeffs(precision, coef, bx, by, nx, ny, bc, kappa, cxx, cxy, nullptr, nullptr, cyy, cyx, s,
+                               may_chain(s));
         for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
-            lx.args.chained = k > 0;  // (the first update follows the coefficients' kernel plainly)
             e = lx.launch(precision, s);
             if (e == cudaSuccess) e = ly.launch(precision, s);
         }

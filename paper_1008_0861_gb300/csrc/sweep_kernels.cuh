@@ -35,6 +35,49 @@
 
 namespace aniso {
 
+// --------------------------------------------------- chained launches
+//
+// Programmatic dependent launch: a kernel launched chained may start while the
+// one before it in the stream still runs.  It waits here, before it first
+// touches memory that others write, and then lets the next one start.  (Both
+// are no-ops in a plain launch.)
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A pointer whose read-only loads must not be moved before the wait (the
+// compiler may take them for invariant otherwise).
+template <typename T> __device__ __forceinline__ void after_wait(const T *&p) { asm volatile("" : "+l"(p)); }
+// Host: a launch of kern(a...), chained or plain, in clusters of `cluster` blocks (0: none).
+template <typename... P, typename... A>
+static cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool chained,
+                                 int cluster, A... a)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[2];
+    unsigned n = 0;
+    if (cluster > 0) {
+        at[n].id = cudaLaunchAttributeClusterDimension;
+        at[n].val.clusterDim.x = (unsigned)cluster;
+        at[n].val.clusterDim.y = 1;
+        at[n].val.clusterDim.z = 1;
+        ++n;
+    }
+    if (chained) {
+        at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[n].val.programmaticStreamSerializationAllowed = 1;
+        ++n;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(a)...);
+}
+
 // ------------------------------------------------------------ arithmetic
 
 template <typename R> struct Num;
@@ -830,11 +873,14 @@ __device__ __forceinline__ void face_coef(B bn0, B bn1, B bt0, B bt1, double kap
 // column from the natural order, every 4-byte store was a sector of its own.
 // 1024^2 FP32: 64 us a call with both, 8 now.
 template <typename B, typename C>
-__global__ void __launch_bounds__(256) face_coeffs_kernel(const B *__restrict__ bx, const B *__restrict__ by, int nx,
+__global__ void __launch_bounds__(256) face_coeffs_kernel(const B *bx, const B *by, int nx,
                                                           int ny, int bc, double kappa, C *cxx, C *cxy, C *cyy, C *cyx,
                                                           C *cyyT, C *cyxT)
 {
     __shared__ C tyy[32][33], tyx[32][33];
+    chain_wait();
+    after_wait(bx);
+    after_wait(by);
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
     const int i = i0 + threadIdx.x;
     const bool per = bc == 1;  // otherwise the boundary faces carry no flux
@@ -845,10 +891,10 @@ __global__ void __launch_bounds__(256) face_coeffs_kernel(const B *__restrict__ 
             const size_t o = (size_t)j * nx + i;
             const size_t ox = i + 1 < nx ? o + 1 : o - (nx - 1);
             const size_t oy = j + 1 < ny ? o + nx : (size_t)i;
-            const B x0 = bx[o], y0 = by[o];
+            const B x0 = __ldg(bx + o), y0 = __ldg(by + o);
             C vxx = C(0.f), vxy = C(0.f), vyy = C(0.f), vyx = C(0.f);
-            if (per || i != nx - 1) face_coef<B, C>(x0, bx[ox], y0, by[ox], kappa, vxx, vxy);
-            if (per || j != ny - 1) face_coef<B, C>(y0, by[oy], x0, bx[oy], kappa, vyy, vyx);
+            if (per || i != nx - 1) face_coef<B, C>(x0, __ldg(bx + ox), y0, __ldg(by + ox), kappa, vxx, vxy);
+            if (per || j != ny - 1) face_coef<B, C>(y0, __ldg(by + oy), x0, __ldg(bx + oy), kappa, vyy, vyx);
             cxx[o] = vxx;
             cxy[o] = vxy;
             if (cyy) {

@@ -242,30 +242,27 @@ cudaError_t launch_line2(int prec, int coef_fp16, const Line2Args &a, int nblock
 }
 
 template <typename B, typename C>
-static void face_launch(const void *bx, const void *by, int nx, int ny, int bc, double kappa, void *cxx,
-                        void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s)
+static cudaError_t face_launch(const void *bx, const void *by, int nx, int ny, int bc, double kappa, void *cxx,
+                               void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s, bool chained)
 {
-    dim3 block(32, 8), grid((nx + 31) / 32, (ny + 31) / 32);
-    face_coeffs_kernel<B, C><<<grid, block, 0, s>>>(
-        static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, kappa, static_cast<C *>(cxx),
-        static_cast<C *>(cxy), static_cast<C *>(cyy), static_cast<C *>(cyx), static_cast<C *>(cyyT),
-        static_cast<C *>(cyxT));
+    return launch_kernel(face_coeffs_kernel<B, C>, dim3((nx + 31) / 32, (ny + 31) / 32), dim3(32, 8), 0, s, chained, 0,
+                         static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, kappa,
+                         static_cast<C *>(cxx), static_cast<C *>(cxy), static_cast<C *>(cyy), static_cast<C *>(cyx),
+                         static_cast<C *>(cyyT), static_cast<C *>(cyxT));
 }
 
-cudaError_t launch_face_coeffs(int bprec, int coef, const void *bx, const void *by, int nx, int ny,
-                               int bc, double kappa, void *cxx, void *cxy, void *cyy, void *cyx,
-                               void *cyyT, void *cyxT, cudaStream_t s)
+cudaError_t launch_face_coeffs(int bprec, int coef, const void *bx, const void *by, int nx, int ny, int bc, double kappa,
+                               void *cxx, void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s,
+                               bool chained)
 {
-    if (bprec == PREC_FP64) {
-        if (coef == 0) face_launch<double, double>(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
-        else if (coef == 1) face_launch<double, float>(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
-        else face_launch<double, __half>(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
-    } else {
-        if (coef == 0) face_launch<float, double>(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
-        else if (coef == 1) face_launch<float, float>(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
-        else face_launch<float, __half>(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
-    }
-    return cudaGetLastError();
+    auto go = [&](auto launch) {
+        return launch(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s, chained);
+    };
+    if (bprec == PREC_FP64)
+        return coef == 0   ? go(face_launch<double, double>)
+               : coef == 1 ? go(face_launch<double, float>)
+                           : go(face_launch<double, __half>);
+    return coef == 0 ? go(face_launch<float, double>) : coef == 1 ? go(face_launch<float, float>) : go(face_launch<float, __half>);
 }
 
 cudaError_t launch_transpose(int elem_bytes, const void *in, void *out, int rows, int cols,

@@ -43,3 +43,38 @@ def test_calls_of_one_step_back_to_back(lib):
     finally:
         a.close()
         b.close()
+
+
+@pytest.mark.parametrize("nx,ny,prec", [(64, 48, FP32), (51, 33, FP32), (50, 50, FP64), (1024, 256, FP32)])
+def test_fields_that_change_every_call(lib, nx, ny, prec):
+    """Set a field, take one step, set another, and so on without a wait: each
+    step sees its own field (the coefficients are rewritten between launches that
+    overlap), as with a wait after every call."""
+    import torch
+    fields = [W.random_instance(nx, ny, seed=k, dt_factor=50.0) for k in range(3)]
+    dt = torch.float64 if prec == FP64 else torch.float32
+    b = [[torch.tensor(v, dtype=dt, device="cuda") for v in (f.bx, f.by)] for f in fields]
+    got = []
+    for wait in (False, True):
+        g = GpuGrid(lib, fields[0], prec)
+        t = g.T.clone()
+        try:
+            for k in range(30):
+                bx, by = b[k % 3]
+                lib.aniso_set_field(g.h, bx, by)
+                if wait:
+                    torch.cuda.synchronize()
+                lib.aniso_step(g.h, g.T, fields[0].dt, 1)
+                if wait:
+                    torch.cuda.synchronize()
+                f = fields[0]
+                if nx * ny <= 1 << 17:
+                    lib.aniso_step_noalloc(nx, ny, f.dx, f.dy, f.chi_par, 0.0, f.bc, prec, by, bx, t, f.dt, 1)
+                    if wait:
+                        torch.cuda.synchronize()
+            lib.aniso_sync(g.h)
+            got.append((g.T.cpu(), t.cpu()))
+        finally:
+            g.close()
+    for x, y in zip(*got):
+        assert torch.equal(x, y)
