@@ -32,24 +32,35 @@ static cudaError_t run7(Kern kern, const Line2Args &a, int cs, size_t smem, cuda
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     const int groups = (a.one.nlines + L7_LPB - 1) / L7_LPB;
-    // (a is never chained here: launches of 100 us and more gain nothing, 4096^2 lost 0.4 %)
+    // (never chained: launches of 100 us and more gain nothing, 4096^2 lost 0.4 %)
     return launch_line_kernel(kern, a, groups * cs, L7_THREADS, smem, s, cs);
 }
 
-template <bool K, bool TM, bool TO>
-static cudaError_t launch7k(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
+// Segments of 8 chunks (pieces of 2048 cells) or 4 (1024), each its own kernel
+// with every loop unrolled.  us a pass with the run-time segment length / with
+// this: 4096^2 FP32, 4 steps 845 / 750 (FP16 coefficients 745 / 666); 8192^2,
+// 2 steps 1585 / 1447; compensated with FP16 coefficients 2279 / 2188; 1024^2
+// compensated, 4 steps 107 / 101.
+template <bool K, bool TM, bool TO, int U>
+static cudaError_t launch7u(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
 {
     const bool vl = a.limiter == LIM_VANLEER;
     if (coef_fp16)
-        return vl ? run7(line7_kernel<__half, true, K, TM, TO>, a, cs, smem, s)
-                  : run7(line7_kernel<__half, false, K, TM, TO>, a, cs, smem, s);
-    return vl ? run7(line7_kernel<float, true, K, TM, TO>, a, cs, smem, s)
-              : run7(line7_kernel<float, false, K, TM, TO>, a, cs, smem, s);
+        return vl ? run7(line7_kernel<__half, true, K, TM, TO, U>, a, cs, smem, s)
+                  : run7(line7_kernel<__half, false, K, TM, TO, U>, a, cs, smem, s);
+    return vl ? run7(line7_kernel<float, true, K, TM, TO, U>, a, cs, smem, s)
+              : run7(line7_kernel<float, false, K, TM, TO, U>, a, cs, smem, s);
+}
+template <bool K, bool TM, bool TO>
+static cudaError_t launch7k(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
+{
+    return a.one.n / cs == 2048 ? launch7u<K, TM, TO, 8>(coef_fp16, a, cs, smem, s)
+                                : launch7u<K, TM, TO, 4>(coef_fp16, a, cs, smem, s);
 }
 
 cudaError_t launch_line7(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
 {
-    if (a.jobs || a.one.n % cs != 0) return cudaErrorInvalidValue;
+    if (a.jobs || (a.one.n != 2048 * cs && a.one.n != 1024 * cs)) return cudaErrorInvalidValue;
     const bool k = a.one.TinLo != nullptr;
     if (k && (!a.one.ToutLo)) return cudaErrorInvalidValue;
     // with args.tmem: the plain state keeps gamma and T_old in tensor memory

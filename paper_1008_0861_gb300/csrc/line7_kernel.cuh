@@ -132,7 +132,11 @@ constexpr int L7_PUB = 16;   // numbers a warp publishes for the interface syste
 // three blocks fit an SM.  TO: each lane's chunks of T_old (hi and lo with K)
 // wait in its TMEM lane from the flux phase to phase C instead of being read
 // again (TM implies it).
-template <typename C, bool VL, bool K, bool TM, bool TO = TM>
+// U: chunks of a lane's segment, 8 (np = 2048) or 4 (np = 1024).  With it fixed
+// every loop over a segment or over the coalesced rounds is unrolled, shared
+// addresses are a lane's base and an immediate, and nothing is copied from one
+// round's registers to the next's (figures in kernels_line7.cu).
+template <typename C, bool VL, bool K, bool TM, bool TO = TM, int U = 8>
 __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args args)
 {
     typedef float R;
@@ -150,7 +154,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     const Line2Job &J = args.one;
     const int lim = args.limiter;
     const int CS = (int)cl_size(), rk = (int)cl_rank();
-    const int n = J.n, np = n / CS, m = np / N, nl = J.nlines;
+    constexpr int V = U, m = P * U, np = m * N;  // chunk rounds of the coalesced phases; chunks and cells of a piece
+    const int n = J.n, nl = J.nlines;
     const int G = WPL * CS;  // interface unknowns of a line
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int lb = warp / WPL, wl = warp - lb * WPL;
@@ -180,10 +185,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     const R lam = (R)J.lam, mu = (R)J.mu;
     const unsigned full = 0xffffffffu;
 
-    const int U = m / P;  // chunks of a lane's segment (m is a multiple of P)
-    const int c_lo = t * U;
-    const int V = U;      // chunk rounds of the coalesced phases
-    const int mfull = m & ~7, logU = 31 - __clz(U);
+    constexpr int LOGU = U == 8 ? 3 : 2;
+    static_assert(U == (1 << LOGU), "segments of 8 or 4 chunks");
     constexpr int NARR = TM ? 2 : 3;                                     // shared arrays a line
     VT *sA = reinterpret_cast<VT *>(smem_raw) + (size_t)lb * NARR * m;  // F -> rho -> delta -> T_new (hi)
     VT *sB = sA + m;                                                     // lam*g -> alpha -> (K) T_new lo
@@ -204,7 +207,10 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
         if (warp == 0) tm_alloc(&s_tmem, TM7_COLS);
         tm_fence_before();
     }
-    auto swz = [mfull, logU](int c) { return c < mfull ? c ^ ((c >> logU) & 7) : c; };
+    // chunk c of a line at c ^ ((c >> LOGU) & 7).  Chunk v P + t of a coalesced
+    // round: v P + cz.  Chunk t U + u of lane t's segment: wz ^ u (t U has no
+    // bits below U, and c >> LOGU is t).
+    const int cz = t ^ ((t >> LOGU) & 7), wz = (t * U) ^ (t & 7);
 
     // The block's rows of this piece into L2 (a hint): input lines line0 - 1
     // .. line0 + 4 (clamped) and the four lines' coefficients.
@@ -254,7 +260,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
             x.g = ld_raw(Gl + p0 + (size_t)c * N);
             x.e = ld_raw(El + p0 + (size_t)c * N);
             x.nc = x.nd = x.nu = x.ncl = x.ndl = x.nul = R(0);
-            if (lane == 31 || c == m - 1) {
+            if (lane == 31) {
                 size_t q = p0 + (size_t)N * (c + 1);
                 if (q >= (size_t)n) q = J.per_line ? 0 : n - 1;
                 q = si(q);
@@ -270,7 +276,6 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
             return x;
         };
         auto body = [&](const In &x, int v) {
-            const int c = v * P + t;
             R Tc[N], Td[N], Tu[N], Tcl[N], Tdl[N], Tul[N], Gv[N], Ev[N];
             V16<R>::unpack(x.c, Tc);
             V16<R>::unpack(x.d, Td);
@@ -295,7 +300,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 vv[j] = level<R, VL>(lim, dif7<K>(Tu[j], Tul[j], Tc[j], Tcl[j]), dif7<K>(Tc[j], Tcl[j], Td[j], Tdl[j]));
             R nT = __shfl_down_sync(full, Tc[0], 1), nTl = K ? __shfl_down_sync(full, Tcl[0], 1) : R(0);
             R nv = __shfl_down_sync(full, vv[0], 1);
-            if (lane == 31 || c == m - 1) {
+            if (lane == 31) {
                 nT = x.nc;
                 nTl = x.ncl;
                 nv = level<R, VL>(lim, dif7<K>(x.nu, x.nul, x.nc, x.ncl), dif7<K>(x.nc, x.ncl, x.nd, x.ndl));
@@ -308,35 +313,22 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 lg[j] = __fmul_rn(lam, Gv[j]);
                 F[j] = flux7<VL>(lim, lg[j], __fmul_rn(mu, Ev[j]), dif7<K>(Tnx, Tnxl, Tc[j], Tcl[j]), vv[j], vnx);
             }
-            sA[swz(c)] = V16<R>::pack(F);
-            sB[swz(c)] = V16<R>::pack(lg);
+            sA[v * P + cz] = V16<R>::pack(F);
+            sB[v * P + cz] = V16<R>::pack(lg);
         };
-        if (K) {  // one round ahead (twice the loads a round)
-            In cur = load(V - 1);
-            if (TO) {  // the block's TMEM address, the first loads in flight
-                __syncthreads();
-                tm_fence_after();
-                tm_lane = s_tmem + ((unsigned)(32 * (warp & 3)) << 16) + 64u * (unsigned)(warp >> 2);
-            }
-            for (int v = V - 1; v >= 0; --v) {
-                const In x = cur;
-                if (v >= 1) cur = load(v - 1);
-                body(x, v);
-            }
-        } else {  // two rounds ahead
-            In cur = load(V - 1);
-            In nxt = V >= 2 ? load(V - 2) : cur;
-            if (TO) {  // the block's TMEM address, the first loads in flight
-                __syncthreads();
-                tm_fence_after();
-                tm_lane = s_tmem + ((unsigned)(32 * (warp & 3)) << 16) + 64u * (unsigned)(warp >> 2);
-            }
-            for (int v = V - 1; v >= 0; --v) {
-                const In x = cur;
-                cur = nxt;
-                if (v >= 2) nxt = load(v - 2);
-                body(x, v);
-            }
+        // the next round's loads in flight (two rounds' took the FP32 tensor-memory
+        // form from 750 to 944 us at 4096^2: spills)
+        In nxt = load(V - 1);
+        if (TO) {  // the block's TMEM address, the first loads in flight
+            __syncthreads();
+            tm_fence_after();
+            tm_lane = s_tmem + ((unsigned)(32 * (warp & 3)) << 16) + 64u * (unsigned)(warp >> 2);
+        }
+#pragma unroll
+        for (int v = V - 1; v >= 0; --v) {
+            const In x = nxt;
+            if (v >= 1) nxt = load(v - 1);
+            body(x, v);
         }
         // the face before the piece: cells q = p0 - 1 (wrapping) and p0
         if (t == 0) {
@@ -383,11 +375,11 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     {
 #pragma unroll
         for (int v = 0; v < N; ++v) ro[v] = ao[v] = go[v] = R(0);
+#pragma unroll
         for (int u = U - 1; u >= 0; --u) {
-            const int c = c_lo + u;
             R F[N], lg[N], co[N], cao[N], cgo[N];
-            V16<R>::unpack(sA[swz(c)], F);
-            V16<R>::unpack(sB[swz(c)], lg);
+            V16<R>::unpack(sA[wz ^ u], F);
+            V16<R>::unpack(sB[wz ^ u], lg);
             if (u == U - 1) {
                 ae = -lg[N - 2];
                 ce = -lg[N - 1];
@@ -400,10 +392,10 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 for (int j = N - 2; j >= 1; --j) elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             } else {
                 elim(Fpend, F[N - 1], lgpend, lg[N - 1], ro[0], ao[0], go[0]);
-                sA[swz(c + 1)] = V16<R>::pack(ro);
-                sB[swz(c + 1)] = V16<R>::pack(ao);
+                sA[wz ^ (u + 1)] = V16<R>::pack(ro);
+                sB[wz ^ (u + 1)] = V16<R>::pack(ao);
                 if (TM) tm_st4(tm_lane + 4u * (unsigned)(u + 1), go[0], go[1], go[2], go[3]);  // warp-wide
-                else sC[swz(c + 1)] = V16<R>::pack(go);
+                else sC[wz ^ (u + 1)] = V16<R>::pack(go);
 #pragma unroll
                 for (int j = N - 1; j >= 1; --j) elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
             }
@@ -424,13 +416,13 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
         const R Fb = t > 0 ? s_ex[lb][0][t - 1] : s_fb[lb][0];
         const R lgb = t > 0 ? s_ex[lb][1][t - 1] : s_fb[lb][1];
         elim(Fpend, Fb, lgpend, lgb, ro[0], ao[0], go[0]);
-        sA[swz(c_lo)] = V16<R>::pack(ro);
-        sB[swz(c_lo)] = V16<R>::pack(ao);
+        sA[wz] = V16<R>::pack(ro);
+        sB[wz] = V16<R>::pack(ao);
         if (TM) {
             tm_st4(tm_lane, go[0], go[1], go[2], go[3]);
             tm_wait_st();  // the recovery reads these columns back
         } else {
-            sC[swz(c_lo)] = V16<R>::pack(go);
+            sC[wz] = V16<R>::pack(go);
         }
     }
 
@@ -469,6 +461,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
             q.U = R(0);
             q.Rr = R(0);
         }
+#pragma unroll
         for (int h = 1; h < 32; h <<= 1) {
             const int tm = (lane - h) & 31, tp = (lane + h) & 31;
             const R iD = Fast<R>::rcp(q.D);
@@ -561,20 +554,20 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     CSum<R> acc;
     {
         R dprev = Xm;
+#pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int c = c_lo + u;
             R r4[N], a4[N], g4[N], d[N];
-            V16<R>::unpack(sA[swz(c)], r4);
-            V16<R>::unpack(sB[swz(c)], a4);
+            V16<R>::unpack(sA[wz ^ u], r4);
+            V16<R>::unpack(sB[wz ^ u], a4);
             if (TM) tm_ld4(tm_lane + 4u * (unsigned)u, g4);  // warp-wide
-            else V16<R>::unpack(sC[swz(c)], g4);
+            else V16<R>::unpack(sC[wz ^ u], g4);
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 d[j] = (u == U - 1 && j == N - 1) ? X : r4[j] - a4[j] * dprev - g4[j] * X;
                 dprev = d[j];
                 if (K) acc.add(d[j]);
             }
-            sA[swz(c)] = V16<R>::pack(d);
+            sA[wz ^ u] = V16<R>::pack(d);
         }
     }
 
@@ -624,6 +617,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
 
     // ---- C: T_new = T_old + delta, coalesced; staged for the store
     bool bad = false;
+#pragma unroll
     for (int v = 0; v < V; ++v) {
         const int c = v * P + t;
         R to[N], tol[N], d[N];
@@ -640,7 +634,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 if (K) pre1l = vcCl[vi(q0 + c + 2 * P)];
             }
         }
-        V16<R>::unpack(sA[swz(c)], d);
+        V16<R>::unpack(sA[v * P + cz], d);
         R hi[N], lo[N];
         R sum = R(0);
 #pragma unroll
@@ -664,8 +658,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 if (K) reinterpret_cast<VT *>(static_cast<R *>(J.ToutLo) + (size_t)lc * n + p0)[c] = V16<R>::pack(lo);
             }
         } else {
-            sA[swz(c)] = V16<R>::pack(hi);
-            if (K) sB[swz(c)] = V16<R>::pack(lo);
+            sA[v * P + cz] = V16<R>::pack(hi);
+            if (K) sB[v * P + cz] = V16<R>::pack(lo);
         }
     }
 
@@ -674,41 +668,46 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     // sector (two neighbouring threads)
     if (J.transpose_out && ilv_out) {
         __syncthreads();
-        R *out = static_cast<R *>(J.Tout);
-        for (int idx = threadIdx.x; idx < 2 * np; idx += blockDim.x) {
-            const int p = idx >> 1, half = idx & 1;
-            const int sc = swz(p >> 2), j = p & 3;
+        // thread: position (tid >> 1) + 128 k of the piece, half (tid & 1) of the pair
+        const int half = threadIdx.x & 1, j = (threadIdx.x >> 1) & 3;
+        const R *src = reinterpret_cast<const R *>(smem_raw) + half * m * N + j;
+        R *dst = static_cast<R *>(J.Tout) + (p0 + (threadIdx.x >> 1)) * 2 * nl + 2 * (size_t)line0 + N * half;
+        const size_t step = (size_t)(L7_THREADS / 2) * 2 * nl;
+#pragma unroll 4
+        for (int k = 0; k < 2 * np / L7_THREADS; ++k, dst += step) {
+            const int c = (threadIdx.x >> 3) + (L7_THREADS / 8) * k;
+            const int sc = (c ^ ((c >> LOGU) & 7)) * N;
             R o[N];
 #pragma unroll
-            for (int i = 0; i < N; ++i)
-                o[i] = reinterpret_cast<const R *>(reinterpret_cast<const VT *>(smem_raw) + (size_t)i * NARR * m +
-                                                   (size_t)half * m + sc)[j];
-            *reinterpret_cast<VT *>(out + (size_t)(p0 + p) * 2 * nl + 2 * (size_t)line0 + N * half) = V16<R>::pack(o);
+            for (int i = 0; i < N; ++i) o[i] = src[i * NARR * m * N + sc];
+            *reinterpret_cast<VT *>(dst) = V16<R>::pack(o);
         }
     } else if (J.transpose_out) {
         __syncthreads();
-        R *out = static_cast<R *>(J.Tout);
-        R *outl = static_cast<R *>(J.ToutLo);
-        const bool vec_ok = (nl & 3) == 0;
-        for (int p = threadIdx.x; p < np; p += blockDim.x) {
-            const int sc = swz(p >> 2), j = p & 3;
+        // thread: position tid + 256 k of the piece
+        const int c0 = threadIdx.x >> 2;
+        const R *src = reinterpret_cast<const R *>(smem_raw) + (c0 ^ ((c0 >> LOGU) & 7)) * N + (threadIdx.x & 3);
+        const size_t row0 = (p0 + threadIdx.x) * nl + line0, step = (size_t)L7_THREADS * nl;
+        R *out = static_cast<R *>(J.Tout) + row0, *outl = static_cast<R *>(J.ToutLo) + (K ? row0 : 0);
+        const bool vec_ok = (nl & 3) == 0 && line0 + N <= nl;
+#pragma unroll
+        for (int k = 0; k < np / L7_THREADS; ++k, out += step, outl += K ? step : 0) {
+            // (256 cells on: 64 chunks, the same swizzle)
             R o[N], ol[N];
 #pragma unroll
             for (int i = 0; i < N; ++i) {
-                const VT *base = reinterpret_cast<const VT *>(smem_raw) + (size_t)i * NARR * m;
-                o[i] = reinterpret_cast<const R *>(base + sc)[j];
-                if (K) ol[i] = reinterpret_cast<const R *>(base + m + sc)[j];
+                o[i] = src[i * NARR * m * N + k * L7_THREADS];
+                if (K) ol[i] = src[(i * NARR + 1) * m * N + k * L7_THREADS];
             }
-            const size_t row = (size_t)(p0 + p) * nl + line0;
-            if (vec_ok && line0 + N <= nl) {
-                *reinterpret_cast<VT *>(out + row) = V16<R>::pack(o);
-                if (K) *reinterpret_cast<VT *>(outl + row) = V16<R>::pack(ol);
+            if (vec_ok) {
+                *reinterpret_cast<VT *>(out) = V16<R>::pack(o);
+                if (K) *reinterpret_cast<VT *>(outl) = V16<R>::pack(ol);
             } else {
 #pragma unroll
                 for (int i = 0; i < N; ++i)
                     if (line0 + i < nl) {
-                        out[row + i] = o[i];
-                        if (K) outl[row + i] = ol[i];
+                        out[i] = o[i];
+                        if (K) outl[i] = ol[i];
                     }
             }
         }
