@@ -5,25 +5,33 @@
 
 namespace aniso {
 
-// n = CS * np with np = 2048 (or 1024 when n is not a multiple of 2048) and
-// CS = 1, 2, 4 or 8 blocks a cluster; four lines a block.
+// n = CS * np with CS = 1, 2, 4 or 8 blocks a cluster.  The plain state in its
+// tensor-memory form (tmem): np = 1024 and eight lines a block up to 8192
+// cells.  Otherwise, and for 16384: np = 2048 (1024 when n is not a multiple of
+// it) and four lines.
+static int pieces7(int n, bool tmem, int *np)
+{
+    *np = tmem && n <= 8192 ? 1024 : n % 2048 == 0 ? 2048 : 1024;
+    if (n % *np != 0) return 0;
+    const int c = n / *np;
+    return c == 1 || c == 2 || c == 4 || c == 8 ? c : 0;
+}
 bool line7_config(int prec, int coef_fp16, int n, int *cs, int *nthreads, size_t *smem, bool tmem)
 {
     if (prec != PREC_FP32 || n <= 0) return false;
     (void)coef_fp16;
-    int np = 2048;
-    if (n % np != 0) np = 1024;
-    if (n % np != 0) return false;
-    const int c = n / np;
-    if (c != 1 && c != 2 && c != 4 && c != 8) return false;
+    int np;
+    const int c = pieces7(n, tmem, &np);
+    if (!c) return false;
+    const int lines = tmem && np == 1024 ? 8 : 4;
     *cs = c;
     *nthreads = L7_THREADS;
-    *smem = (size_t)L7_LPB * (tmem ? 2 : 3) * (size_t)(np / 4) * 16;
+    *smem = (size_t)lines * (tmem ? 2 : 3) * (size_t)(np / 4) * 16 + (lines == 8 ? 64 : 0);
     return true;
 }
 
 template <typename Kern>
-static cudaError_t run7(Kern kern, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
+static cudaError_t run7(Kern kern, const Line2Args &a, int lines, int cs, size_t smem, cudaStream_t s)
 {
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, kern);
@@ -31,7 +39,7 @@ static cudaError_t run7(Kern kern, const Line2Args &a, int cs, size_t smem, cuda
     if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
-    const int groups = (a.one.nlines + L7_LPB - 1) / L7_LPB;
+    const int groups = (a.one.nlines + lines - 1) / lines;
     // (never chained: launches of 100 us and more gain nothing, 4096^2 lost 0.4 %)
     return launch_line_kernel(kern, a, groups * cs, L7_THREADS, smem, s, cs);
 }
@@ -41,21 +49,26 @@ static cudaError_t run7(Kern kern, const Line2Args &a, int cs, size_t smem, cuda
 // this: 4096^2 FP32, 4 steps 845 / 750 (FP16 coefficients 745 / 666); 8192^2,
 // 2 steps 1585 / 1447; compensated with FP16 coefficients 2279 / 2188; 1024^2
 // compensated, 4 steps 107 / 101.
-template <bool K, bool TM, bool TO, int U>
+template <bool K, bool TM, bool TO, int U, int WPL>
 static cudaError_t launch7u(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
 {
     const bool vl = a.limiter == LIM_VANLEER;
+    constexpr int L = L7_THREADS / (32 * WPL);
     if (coef_fp16)
-        return vl ? run7(line7_kernel<__half, true, K, TM, TO, U>, a, cs, smem, s)
-                  : run7(line7_kernel<__half, false, K, TM, TO, U>, a, cs, smem, s);
-    return vl ? run7(line7_kernel<float, true, K, TM, TO, U>, a, cs, smem, s)
-              : run7(line7_kernel<float, false, K, TM, TO, U>, a, cs, smem, s);
+        return vl ? run7(line7_kernel<__half, true, K, TM, TO, U, WPL>, a, L, cs, smem, s)
+                  : run7(line7_kernel<__half, false, K, TM, TO, U, WPL>, a, L, cs, smem, s);
+    return vl ? run7(line7_kernel<float, true, K, TM, TO, U, WPL>, a, L, cs, smem, s)
+              : run7(line7_kernel<float, false, K, TM, TO, U, WPL>, a, L, cs, smem, s);
 }
 template <bool K, bool TM, bool TO>
 static cudaError_t launch7k(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)
 {
-    return a.one.n / cs == 2048 ? launch7u<K, TM, TO, 8>(coef_fp16, a, cs, smem, s)
-                                : launch7u<K, TM, TO, 4>(coef_fp16, a, cs, smem, s);
+    if constexpr (TM)
+        return a.one.n / cs == 2048 ? launch7u<K, TM, TO, 8, 2>(coef_fp16, a, cs, smem, s)
+                                    : launch7u<K, TM, TO, 8, 1>(coef_fp16, a, cs, smem, s);
+    else
+        return a.one.n / cs == 2048 ? launch7u<K, TM, TO, 8, 2>(coef_fp16, a, cs, smem, s)
+                                    : launch7u<K, TM, TO, 4, 2>(coef_fp16, a, cs, smem, s);
 }
 
 cudaError_t launch_line7(int coef_fp16, const Line2Args &a, int cs, size_t smem, cudaStream_t s)

@@ -121,10 +121,7 @@ template <bool K> __device__ __forceinline__ float dif7(float ah, float al, floa
     return K ? __fadd_rn(__fsub_rn(ah, bh), __fsub_rn(al, bl)) : __fsub_rn(ah, bh);
 }
 
-constexpr int L7_P = 64;     // lanes of a line's team in a block
-constexpr int L7_WPL = 2;    // warps of a team
-constexpr int L7_LPB = 4;    // lines a block holds
-constexpr int L7_THREADS = L7_P * L7_LPB;
+constexpr int L7_THREADS = 256;  // lines a block holds x lanes of a line's team
 constexpr int L7_PUB = 16;   // numbers a warp publishes for the interface system
 
 // TM: each lane's gamma goes to its own tensor-memory lane instead of shared
@@ -136,12 +133,18 @@ constexpr int L7_PUB = 16;   // numbers a warp publishes for the interface syste
 // every loop over a segment or over the coalesced rounds is unrolled, shared
 // addresses are a lane's base and an immediate, and nothing is copied from one
 // round's registers to the next's (figures in kernels_line7.cu).
-template <typename C, bool VL, bool K, bool TM, bool TO = TM, int U = 8>
+// WPL: warps of a line's team in a block.  2: four lines a block, pieces of
+// 2048 (or 1024) cells, 16 bytes a position in the transposed store.  1: eight
+// lines and pieces of 1024 cells, so that the store writes whole 32-byte sectors
+// (4096^2 750 -> 717 us for 4 steps, 8192^2 unchanged; leaving the store out
+// altogether saves 22 and 29 %, a line-major store costs nothing).  The lanes'
+// segments, and so all arithmetic, are the same.
+template <typename C, bool VL, bool K, bool TM, bool TO = TM, int U = 8, int WPL = 2>
 __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args args)
 {
     typedef float R;
     typedef float4 VT;
-    constexpr int N = 4, P = L7_P, WPL = L7_WPL, LPB = L7_LPB;
+    constexpr int N = 4, P = 32 * WPL, LPB = L7_THREADS / P;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ __align__(16) float s_pub[LPB][WPL][L7_PUB];  // per warp: the interface system's inputs
     __shared__ float s_b[LPB][32];             // interface unknowns b_g of each line
@@ -188,7 +191,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     constexpr int LOGU = U == 8 ? 3 : 2;
     static_assert(U == (1 << LOGU), "segments of 8 or 4 chunks");
     constexpr int NARR = TM ? 2 : 3;                                     // shared arrays a line
-    VT *sA = reinterpret_cast<VT *>(smem_raw) + (size_t)lb * NARR * m;  // F -> rho -> delta -> T_new (hi)
+    // (the second group of four lines 16 banks on, for the transposed store's half-warps)
+    VT *sA = reinterpret_cast<VT *>(smem_raw) + lb * NARR * m + (lb >> 2) * 4;  // F -> rho -> delta -> T_new (hi)
     VT *sB = sA + m;                                                     // lam*g -> alpha -> (K) T_new lo
     VT *sC = sA + 2 * m;                                                 // gamma (shared-memory form)
     // TMEM forms: warp 0 allocates the block's 128 columns now; the address
@@ -208,13 +212,15 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
         tm_fence_before();
     }
     // chunk c of a line at c ^ ((c >> LOGU) & 7).  Chunk v P + t of a coalesced
-    // round: v P + cz.  Chunk t U + u of lane t's segment: wz ^ u (t U has no
-    // bits below U, and c >> LOGU is t).
-    const int cz = t ^ ((t >> LOGU) & 7), wz = (t * U) ^ (t & 7);
+    // round: v P + (cz ^ key of v P) (v P >> LOGU and t >> LOGU share no bits of
+    // the key).  Chunk t U + u of lane t's segment: wz ^ u (t U has no bits below
+    // U, and c >> LOGU is t).
+    const int cz0 = t ^ ((t >> LOGU) & 7), wz = (t * U) ^ (t & 7);
+    auto cz = [cz0](int v) { return v * P + (cz0 ^ (((v * P) >> LOGU) & 7)); };
 
     // The block's rows of this piece into L2 (a hint): input lines line0 - 1
-    // .. line0 + 4 (clamped) and the four lines' coefficients.
-    if (threadIdx.x < 6) {
+    // .. line0 + LPB (clamped) and the block's lines' coefficients.
+    if (threadIdx.x < LPB + 2) {
         const int l = max(0, min(line0 - 1 + (int)threadIdx.x, nl - 1));
         if (ilv_in) {
             l2_prefetch(Tin + (size_t)l * ls + 2 * p0, 2 * (size_t)np * sizeof(R));
@@ -222,8 +228,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
             l2_prefetch(Tin + (size_t)l * n + p0, (size_t)np * sizeof(R));
             if (K) l2_prefetch(static_cast<const R *>(J.TinLo) + (size_t)l * n + p0, (size_t)np * sizeof(R));
         }
-    } else if (threadIdx.x < 6 + LPB) {
-        const int l = min(line0 + (int)threadIdx.x - 6, nl - 1);
+    } else if (threadIdx.x < LPB + 2 + LPB) {
+        const int l = min(line0 + (int)threadIdx.x - (LPB + 2), nl - 1);
         l2_prefetch(static_cast<const C *>(J.g) + (size_t)l * n + p0, (size_t)np * sizeof(C));
         l2_prefetch(static_cast<const C *>(J.e) + (size_t)l * n + p0, (size_t)np * sizeof(C));
     }
@@ -313,8 +319,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 lg[j] = __fmul_rn(lam, Gv[j]);
                 F[j] = flux7<VL>(lim, lg[j], __fmul_rn(mu, Ev[j]), dif7<K>(Tnx, Tnxl, Tc[j], Tcl[j]), vv[j], vnx);
             }
-            sA[v * P + cz] = V16<R>::pack(F);
-            sB[v * P + cz] = V16<R>::pack(lg);
+            sA[cz(v)] = V16<R>::pack(F);
+            sB[cz(v)] = V16<R>::pack(lg);
         };
         // the next round's loads in flight (two rounds' took the FP32 tensor-memory
         // form from 750 to 944 us at 4096^2: spills)
@@ -634,7 +640,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 if (K) pre1l = vcCl[vi(q0 + c + 2 * P)];
             }
         }
-        V16<R>::unpack(sA[v * P + cz], d);
+        V16<R>::unpack(sA[cz(v)], d);
         R hi[N], lo[N];
         R sum = R(0);
 #pragma unroll
@@ -658,8 +664,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 if (K) reinterpret_cast<VT *>(static_cast<R *>(J.ToutLo) + (size_t)lc * n + p0)[c] = V16<R>::pack(lo);
             }
         } else {
-            sA[v * P + cz] = V16<R>::pack(hi);
-            if (K) sB[v * P + cz] = V16<R>::pack(lo);
+            sA[cz(v)] = V16<R>::pack(hi);
+            if (K) sB[cz(v)] = V16<R>::pack(lo);
         }
     }
 
@@ -681,6 +687,31 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
 #pragma unroll
             for (int i = 0; i < N; ++i) o[i] = src[i * NARR * m * N + sc];
             *reinterpret_cast<VT *>(dst) = V16<R>::pack(o);
+        }
+    } else if (WPL == 1 && J.transpose_out) {
+        __syncthreads();
+        // thread: position 16 w + (lane & 15) + 128 k of the piece, lines 4 (lane >> 4) .. + 3
+        static_assert(WPL == 2 || !K, "one warp a line: the plain state");
+        const int grp = lane >> 4, pp = warp * 16 + (lane & 15);
+        const R *src = reinterpret_cast<const R *>(smem_raw) + grp * (4 * NARR * m + 4) * N + (pp & 3);
+        const int l0 = line0 + 4 * grp;
+        const size_t step = (size_t)(L7_THREADS / 2) * nl;
+        R *out = static_cast<R *>(J.Tout) + (p0 + pp) * nl + l0;
+        const bool vec_ok = (nl & 3) == 0 && l0 + N <= nl;
+#pragma unroll
+        for (int k = 0; k < np / (L7_THREADS / 2); ++k, out += step) {
+            const int c = (pp >> 2) + (L7_THREADS / 8) * k;
+            const int sc = (c ^ ((c >> LOGU) & 7)) * N;
+            R o[N];
+#pragma unroll
+            for (int i = 0; i < N; ++i) o[i] = src[i * NARR * m * N + sc];
+            if (vec_ok) {
+                *reinterpret_cast<VT *>(out) = V16<R>::pack(o);
+            } else {
+#pragma unroll
+                for (int i = 0; i < N; ++i)
+                    if (l0 + i < nl) out[i] = o[i];
+            }
         }
     } else if (J.transpose_out) {
         __syncthreads();
