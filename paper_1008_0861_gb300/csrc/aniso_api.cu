@@ -430,7 +430,10 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
                                 &smem, false, ragged)
                  : line2_config(h->prec, n, transposed, &J.team, &J.lines_per_block, &nthreads, &smem,
                                 h->seg_chunks);
-    if (v4 && ok) J.swz = line4_swizzle(h->prec, n, J.team);
+    if (v4 && ok) {
+        J.swz = line4_swizzle(h->prec, n, J.team);
+        if (!ragged) a.rounds = line4_rounds(h->prec, h->limiter, n, J.team);
+    }
     // lines above line4's limit: the long-line kernels (constant diffusivity
     // only); the compensated state runs on the cluster kernel alone
     if (v4 && in_lo) ok = false;
@@ -1155,6 +1158,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         int diag_region = -1;  // line4 y-update with diagnostics: its partials region
         int tmem = 0;          // line4: gamma in tensor memory
         int ragged = 0;        // line4: the form for any length and alignment
+        int rounds = 0;        // line4: the launch's chunk rounds, where they are the form's constant
         int step = 0;          // the call's step the launch belongs to
     };
     std::vector<unsigned char> blob;
@@ -1264,7 +1268,8 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         struct Cls {
             int occ;
             size_t sm;
-            int form;  // 0 shared memory, 1 tensor memory, 2 ragged
+            int form;    // 0 shared memory, 1 tensor memory, 2 ragged
+            int rounds;  // line4_rounds: the form with that many chunk rounds, or 0
         };
         const bool tm_on = b->hs[0]->tmem != 0 && prec == PREC_FP32;
         std::vector<Cls> cls(jobs.size());
@@ -1278,18 +1283,32 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                 shape_rc = fail(ANISO_ERR_UNSUPPORTED, "batch: line length %d does not fit the block shape", J.n);
             J.swz = line4_swizzle(prec, J.n, J.team);
             int occ = line4_blocks_per_sm(prec, fp16, b->hs[0]->limiter, nthreads, sm, false);
-            cls[k] = {occ > 0 ? occ : 0, sm, ragged(J) ? 2 : 0};
+            const int rounds = ragged(J) ? 0 : line4_rounds(prec, b->hs[0]->limiter, J.n, J.team);
+            cls[k] = {occ > 0 ? occ : 0, sm, ragged(J) ? 2 : 0, rounds};
             int t0, t1, t2;
             size_t smt = 0;
             if (tm_on && !ragged(J) && line4_config(prec, J.n, true, nthreads / 32, seg, &t0, &t1, &t2, &smt, true)) {
                 const int occt = line4_blocks_per_sm(prec, fp16, b->hs[0]->limiter, nthreads, smt, true,
                                                      line4_tm_cols(J.n, J.team));
-                if (occt > cls[k].occ) cls[k] = {occt, smt, 1};
+                if (occt > cls[k].occ) cls[k] = {occt, smt, 1, rounds};
             }
         }
-        // per form, classes in ascending occupancy (largest lines first); at
-        // most three a form, the highest-occupancy ones merged
-        int region = 0;
+        // Where every line of the sweep has the same number of chunk rounds, the
+        // form that has it as a constant (100 grids of 512^2: 1007 -> 939 us for 4
+        // steps, 60 of 896^2 1731 -> 1629).  An uneven batch keeps the run-time
+        // form: a launch for each number lost what the constant won (200 grids up
+        // to 512^2: 686 -> 723 us), as did 8 rounds in tensor memory (spills).
+        for (auto &c : cls)
+            if (c.rounds != cls[0].rounds || (c.rounds == 8 && c.form == 1)) {
+                for (auto &d : cls) d.rounds = 0;
+                break;
+            }
+        // Per form, the classes in ascending occupancy (largest lines first), at
+        // most three, the highest-occupancy ones merged.
+        struct Sel {
+            int form, lo, hi;
+        };
+        std::vector<Sel> sels;
         for (int form : {1, 0, 2}) {
             std::vector<int> occs;
             for (auto &c : cls)
@@ -1298,13 +1317,17 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             occs.erase(std::unique(occs.begin(), occs.end()), occs.end());
             // (merging never drops the lowest class: its range reaches up to the next kept one)
             while ((int)occs.size() > 3) occs.erase(occs.end() - (occs.size() >= 3 ? 2 : 1));
-            for (size_t ci = 0; ci < occs.size(); ++ci) {
-                const int lo = occs[ci], hi = ci + 1 < occs.size() ? occs[ci + 1] : 1 << 30;
+            for (size_t ci = 0; ci < occs.size(); ++ci)
+                sels.push_back({form, occs[ci], ci + 1 < occs.size() ? occs[ci + 1] : 1 << 30});
+        }
+        int region = 0;
+        {
+            for (const Sel &sel : sels) {
                 std::vector<Line2Job> part;
                 size_t smem = 0;
                 int blocks = 0;
                 for (size_t k = 0; k < jobs.size(); ++k) {
-                    if (cls[k].form != form || cls[k].occ < lo || cls[k].occ >= hi) continue;
+                    if (cls[k].form != sel.form || cls[k].occ < sel.lo || cls[k].occ >= sel.hi) continue;
                     Line2Job J = jobs[k];
                     smem = std::max(smem, cls[k].sm);
                     J.block0 = blocks;
@@ -1315,8 +1338,9 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                 if (part.empty()) continue;
                 Launch L{kind_xy == 0 ? 7 : 8, blob.size(), (int)part.size(), blocks, nthreads, smem};
                 L.group = group;
-                L.tmem = form == 1;
-                L.ragged = form == 2;
+                L.tmem = sel.form == 1;
+                L.ragged = sel.form == 2;
+                L.rounds = cls[0].rounds;
                 if (kind_xy == 1 && diag) L.diag_region = region;
                 ++region;
                 const unsigned char *p = reinterpret_cast<const unsigned char *>(part.data());
@@ -1656,6 +1680,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             if (L.table >= 0)
                 a.block_job = reinterpret_cast<const int *>(static_cast<unsigned char *>(b->d_jobs) + L.table);
             a.tmem = L.tmem;
+            a.rounds = L.rounds;
             a.limiter = b->hs[0]->limiter;
             a.err = err;
             auto launch4 = [&](const Line2Args &args) {

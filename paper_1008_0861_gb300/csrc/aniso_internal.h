@@ -135,6 +135,9 @@ struct Line2Args {
     // 1: launched to start while the kernel before it in the stream drains
     // (programmatic dependent launch); in a capture never a call's first launch
     int chained;
+    // line4, FP32 van Leer: the chunk rounds of every line of the launch, 4 to 8
+    // (line4_rounds), to run the form that has them as a constant; 0: any
+    int rounds;
 };
 // Finish the diagnostics of one line4 launch: for every job, the partials of
 // its blocks in block order -> ring[diag_slot] = (sum, min, max).
@@ -183,6 +186,14 @@ cudaError_t launch_line4_ragged(int prec, int coef_fp16, const Line2Args &a, int
                                 cudaStream_t s);
 cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads,
                          size_t smem, cudaStream_t s);
+// Line2Args::rounds for lines of n cells in teams of `team` lanes, or 0.
+int line4_rounds(int prec, int limiter, int n, int team);
+cudaError_t launch_line4_rounds(int coef_fp16, bool alone, const Line2Args &a, int nblocks, int nthreads, size_t smem,
+                                cudaStream_t s);
+cudaError_t launch_line4_rounds_tm(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
+                                   cudaStream_t s);
+cudaError_t launch_line4_rounds_3d(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
+                                   cudaStream_t s);
 // Long lines (line6): FP32 2048 < n <= 4096, FP64 1024 < n <= 4096, teams of
 // 128 lanes over four warps; FP32 `lines` (4 or 2) lines per block, FP64 two.
 // False when the line does not fit.

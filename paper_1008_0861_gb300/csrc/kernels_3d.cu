@@ -116,6 +116,7 @@ cudaError_t launch_line4_3d(int prec, int coef_fp16, const Line2Args &a, int nbl
             return run4_3d(line4_kernel<float, __half, false, true, false, true>, a, nblocks, nthreads, smem, s);
         return run4_3d(line4_kernel<float, float, false, true, false, true>, a, nblocks, nthreads, smem, s);
     }
+    if (prec == PREC_FP32 && a.rounds) return launch_line4_rounds_3d(coef_fp16, a, nblocks, nthreads, smem, s);
     if (coef_fp16)
         return vl ? run4_3d(line4_kernel<float, __half, true, true>, a, nblocks, nthreads, smem, s)
                   : run4_3d(line4_kernel<float, __half, false, true>, a, nblocks, nthreads, smem, s);

@@ -40,12 +40,14 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
         if (prec == PREC_FP64)
             return vl ? run4(line4_kernel<double, double, true, false, true>, a, nblocks, nthreads, smem, s)
                       : run4(line4_kernel<double, double, false, false, true>, a, nblocks, nthreads, smem, s);
+        if (vl && deep && a.rounds) return launch_line4_rounds(0, true, a, nblocks, nthreads, smem, s);
         if (vl && deep)
             return run4(line4_kernel<float, float, true, false, true, false, false, 3>, a, nblocks, nthreads, smem, s);
         return vl ? run4(line4_kernel<float, float, true, false, true>, a, nblocks, nthreads, smem, s)
                   : run4(line4_kernel<float, float, false, false, true>, a, nblocks, nthreads, smem, s);
     }
     if (a.tmem && prec == PREC_FP32) {  // gamma in tensor memory
+        if (a.rounds) return launch_line4_rounds_tm(coef_fp16, a, nblocks, nthreads, smem, s);
         if (coef_fp16)
             return vl ? run4(line4_kernel<float, __half, true, false, false, false, true>, a, nblocks, nthreads, smem, s)
                       : run4(line4_kernel<float, __half, false, false, false, false, true>, a, nblocks, nthreads, smem, s);
@@ -55,6 +57,7 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
     if (prec == PREC_FP64)
         return vl ? run4(line4_kernel<double, double, true>, a, nblocks, nthreads, smem, s)
                   : run4(line4_kernel<double, double, false>, a, nblocks, nthreads, smem, s);
+    if (prec == PREC_FP32 && a.rounds) return launch_line4_rounds(coef_fp16, deep, a, nblocks, nthreads, smem, s);
     if (vl && deep)
         return coef_fp16 ? run4(line4_kernel<float, __half, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s)
                          : run4(line4_kernel<float, float, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s);
@@ -77,6 +80,13 @@ template <typename K> static int occ4(K kern, int nthreads, size_t smem)
     int blocks = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, nthreads, smem) != cudaSuccess) return -1;
     return blocks;
+}
+
+int line4_rounds(int prec, int limiter, int n, int team)
+{
+    if (prec != PREC_FP32 || limiter != LIM_VANLEER || n % 4 != 0) return 0;
+    const int m = n / 4, V = (m + team - 1) / team;
+    return V >= 4 && V <= 8 ? V : 0;
 }
 
 int line4_tm_cols(int n, int team)

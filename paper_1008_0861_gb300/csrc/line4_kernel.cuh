@@ -151,8 +151,9 @@ template <typename R> __device__ __forceinline__ R lim_level(int lim, R a, R b)
 // nonzero); one approximate reciprocal.
 __device__ __forceinline__ float vl_level(float a, float b)
 {
-    const float p = a * b;
-    const float r = (p + p) * frcp_approx(a + b);
+    // (spelled out: a b + p could be fused, and must round alike in all forms)
+    const float p = __fmul_rn(a, b);
+    const float r = __fmul_rn(__fadd_rn(p, p), frcp_approx(__fadd_rn(a, b)));
     return p > 0.f ? r : 0.f;
 }
 template <typename R, bool VL> __device__ __forceinline__ R level(int lim, R a, R b)
@@ -383,6 +384,10 @@ __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sy
 // after it (the wrap or the mirrored ghost), which the last face needs.  The
 // last segment ends at position nv - 1 of its last chunk.  A line's solve is
 // the same as with whole chunks.
+// VC: the chunk rounds V of the launch's lines (their longest segment) as a
+// constant, 0 = from the job.  The loops over rounds and segments are then
+// unrolled: no counters, and nothing moved from one chunk's registers to the
+// next's.
 // IMPL: a purely implicit update (no transverse term, mu = mu2 = 0: the second
 // half-update of each axis in the 4-step scheme); neighbouring lines and
 // transverse coefficients are then neither loaded nor limited.
@@ -392,7 +397,7 @@ __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sy
 // lane's chunks of T_old wait there too, from the flux phase to phase C
 // (4 V + 4 V columns of the block's 32 or 64).
 template <typename R, typename C, bool VL, bool D3 = false, bool NL = false, bool IMPL = false, bool TM = false,
-          int RING = 1, bool RAG = false>
+          int RING = 1, bool RAG = false, int VC = 0>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4) : 2) line4_kernel(Line2Args args)
 {
     static_assert(!TM || (sizeof(R) == 4 && !D3), "TMEM line state: FP32 2-D only");
@@ -480,8 +485,10 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     // segment of lane t: chunks [c_lo, c_lo + Ut); the first rr lanes one more
     const int U = m >> logP, rr = m & (P - 1);
     const int Ut = U + (t < rr ? 1 : 0);
-    const int c_lo = t * U + (t < rr ? t : rr);
-    const int V = U + (rr ? 1 : 0);  // chunk rounds of the coalesced phases
+    const int c_lo = t * U + (t < rr ? t : rr), ce = c_lo + Ut - 1;
+    const int V = VC > 0 ? VC : U + (rr ? 1 : 0);  // chunk rounds of the coalesced phases
+    // (the tensor-memory form by fours: unrolled whole it spilled at 64 registers)
+    constexpr int UNR = VC > 0 ? (TM ? 4 : VC) : 1;
     const int WA = m << logL;        // chunks per array in one warp's area
     const int mfull = m & ~7, logU = 31 - __clz(U);
     constexpr int NARR = TM ? 2 : 3;  // shared arrays per warp area
@@ -561,6 +568,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
             tm_base = s_tmem;
             tm_lane = tm_base + ((unsigned)(32 * (warp & 3)) << 16);
         }
+#pragma unroll UNR
         for (int v0 = V - 1; v0 >= 0; v0 -= RING)
 #pragma unroll
         for (int r = 0; r < RING; ++r) {
@@ -672,19 +680,21 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         bool pend = false;      // RAG: the segment ends in row 0 of its last chunk, whose lower face is still to come
 #pragma unroll
         for (int v = 0; v < N; ++v) ro[v] = ao[v] = go[v] = R(0);
-        // (TMEM form: every lane runs all V rounds, so that the warp-wide TMEM
-        // stores stay uniform; a lane's rounds past its segment do nothing but
-        // store to columns its segment does not use)
-        for (int u = TM ? V - 1 : Ut - 1; u >= 0; --u) {
-            R gs[N];  // gamma of the chunk above once its row 0 is eliminated (TMEM form)
+        // Chunk k = 0, 1, .. counts down from the segment's last, ce: the lanes'
+        // segments differ by one chunk at their other end, so all eliminate their
+        // last chunks together.  (TMEM form: every lane runs all V rounds, so that
+        // the warp-wide stores stay uniform; chunk k's gamma goes to column 4 k.)
+        R gs[N];  // gamma of chunk k - 1 once its row 0 is eliminated (TMEM form)
 #pragma unroll
-            for (int j = 0; j < N; ++j) gs[j] = R(0);
-            if (!TM || u < Ut) {
-            const int c = c_lo + u;
+        for (int j = 0; j < N; ++j) gs[j] = R(0);
+#pragma unroll UNR
+        for (int k = 0; k < (VC > 0 || TM ? V : Ut); ++k) {
+            if ((VC == 0 && !TM) || k < V - 1 || k < Ut) {
+            const int c = ce - k;
             R F[N], lg[N], co[N], cao[N], cgo[N];
             V16<R>::unpack(sA[swz(c)], F);
             V16<R>::unpack(sB[swz(c)], lg);
-            if (RAG && u == Ut - 1 && c == m - 1 && nv < N) {
+            if (RAG && k == 0 && c == m - 1 && nv < N) {
                 // the line's last cell is position nv - 1
                 Flast = F[0];
                 lge = lg[0];
@@ -702,7 +712,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
 #pragma unroll
                 for (int j = N - 2; j >= 1; --j)
                     if (j < nv - 1) sg.elim(F[j], F[j - 1], lg[j], lg[j - 1], co[j], cao[j], cgo[j]);
-            } else if (u == Ut - 1) {
+            } else if (k == 0) {
                 // row e (last cell of the segment) enters the reduced system
                 lge = lg[N - 1];
                 lgem = lg[N - 2];
@@ -740,9 +750,9 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
                 go[j] = cgo[j];
             }
             }
-            // (chunk u + 1's gamma at columns 4 (u + 1); in the first round there is none)
+            // (the last round's, which only the longer segments have, is stored below)
             if constexpr (TM)
-                if (u + 1 < V) tm_st4(tm_lane + 4u * (unsigned)(u + 1), gs[0], gs[1], gs[2], gs[3]);
+                if (k >= 1 && k < V - 1) tm_st4(tm_lane + 4u * (unsigned)(k - 1), gs[0], gs[1], gs[2], gs[3]);
         }
         // row s needs the face below the segment: the previous lane's last face
         const int tp = (t - 1) & (P - 1);
@@ -757,7 +767,12 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         sA[swz(c_lo)] = V16<R>::pack(ro);
         sB[swz(c_lo)] = V16<R>::pack(ao);
         if constexpr (TM) {
-            tm_st4(tm_lane, go[0], go[1], go[2], go[3]);
+            // a segment of V chunks: chunk V - 2 at 4 (V - 2), V - 1 at 4 (V - 1); one of V - 1: V - 2 is its first
+            const bool lng = Ut == V;
+            if (V >= 2)
+                tm_st4(tm_lane + 4u * (unsigned)(V - 2), lng ? gs[0] : go[0], lng ? gs[1] : go[1], lng ? gs[2] : go[2],
+                       lng ? gs[3] : go[3]);
+            tm_st4(tm_lane + 4u * (unsigned)(V - 1), go[0], go[1], go[2], go[3]);
             tm_wait_st();  // the recovery below reads these columns back
         } else {
             sC[swz(c_lo)] = V16<R>::pack(go);
@@ -791,18 +806,19 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     // ---- B2: forward recovery of lane t's segment (delta over rho)
     {
         R dprev = Xm;
-        for (int u = 0; u < (TM ? V : Ut); ++u) {
+#pragma unroll UNR
+        for (int k = (VC > 0 || TM ? V : Ut) - 1; k >= 0; --k) {
             R g4[N];
-            if constexpr (TM) tm_ld4(tm_lane + 4u * (unsigned)u, reinterpret_cast<float *>(g4));  // warp-wide
-            if (TM && u >= Ut) continue;
-            const int c = c_lo + u;
+            if constexpr (TM) tm_ld4(tm_lane + 4u * (unsigned)k, reinterpret_cast<float *>(g4));  // warp-wide
+            if ((VC > 0 || TM) && k == V - 1 && k >= Ut) continue;
+            const int c = ce - k;
             R r4[N], a4[N], d[N];
             V16<R>::unpack(sA[swz(c)], r4);
             V16<R>::unpack(sB[swz(c)], a4);
             if constexpr (!TM) V16<R>::unpack(sC[swz(c)], g4);
 #pragma unroll
             for (int j = 0; j < N; ++j) {
-                d[j] = (u == Ut - 1 && j == N - 1) ? X : r4[j] - a4[j] * dprev - g4[j] * X;
+                d[j] = (k == 0 && j == N - 1) ? X : r4[j] - a4[j] * dprev - g4[j] * X;
                 if (RAG && c == m - 1 && j >= nv - 1) d[j] = j == nv - 1 ? X : R(0);
                 dprev = d[j];
             }
@@ -818,6 +834,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     R dh = R(0), dl = R(0), dmn = R(INFINITY), dmx = R(-INFINITY);
     {
         VT *vout = reinterpret_cast<VT *>(static_cast<R *>(J.Tout) + (size_t)lc * n);
+#pragma unroll UNR
         for (int v = 0; v < V; ++v) {
             const int c = (v << logP) + t;
             R to[N], d[N];

@@ -126,6 +126,7 @@ bool line_launch(int prec, int n, int nlines, const void *in, void *out, const v
     J.per_line = J.per_cross = per;
     J.transpose_out = 1;
     J.swz = line4_swizzle(prec, n, J.team);
+    L->args.rounds = L->ragged ? 0 : line4_rounds(prec, LIM_VANLEER, n, J.team);
     J.nblocks = (nlines + J.lines_per_block - 1) / J.lines_per_block;
     if (prec == PREC_FP32 && !L->ragged) L->smem = line4_smem_alone(J.nblocks, L->smem);
     return true;

@@ -45,3 +45,31 @@ def test_nonlinear_alone(lib, nx, ny):
     finally:
         a.close()
         c.close()
+
+
+# every number of chunk rounds with a form of its own (4 .. 8), whole and uneven
+# segments, teams of 32, 16, 8 and 4 lanes, and the lengths on both sides (3 and 9 rounds)
+@pytest.mark.parametrize("n", [12, 48, 64, 92, 128, 132, 252, 256, 260, 400, 508, 512, 516, 640, 644, 768, 900, 1020, 1024, 1028])
+def test_constant_rounds_equal_run_time_rounds(lib, n):
+    """A grid alone, a batch of one shape and a batch whose other grid has another
+    number of rounds (the run-time form), with and without tensor memory."""
+    import torch
+    inst = W.random_instance(n, 40, seed=n, dt_factor=50.0)
+    other = W.random_instance(96 if n != 96 else 64, 16, seed=1, dt_factor=50.0)
+    want = None
+    for mixed in (False, True):
+        for tmem in (0, 1):
+            gs = [GpuGrid(lib, inst, FP32) for _ in range(2)] + ([GpuGrid(lib, other, FP32)] if mixed else [])
+            s = GpuGrid(lib, inst, FP32)
+            try:
+                lib.aniso_set_option(gs[0].h, lib.ANISO_OPT_TMEM, tmem)
+                b = lib.aniso_batch_create([g.h for g in gs])
+                lib.aniso_step_batched(b, [g.T for g in gs], [g.inst.dt for g in gs], [2] * len(gs))
+                torch.cuda.synchronize()
+                want = s.step(2) if want is None else want
+                for g in gs[:2]:
+                    assert np.array_equal(g.T.double().cpu().numpy(), want)
+                lib.aniso_batch_destroy(b)
+            finally:
+                for g in gs + [s]:
+                    g.close()
