@@ -200,8 +200,11 @@ static int enqueue3(aniso3_ctx *h, int d, const void *in, void *out, double lam,
         return fail(ANISO_ERR_UNSUPPORTED, "3-D line kernel cannot take n=%d", J.n);
     J.swz = line4_swizzle(h->prec, J.n, J.team);
     A.rounds = line4_rounds(h->prec, h->limiter, J.n, J.team);
+    // (unrolled 3-D rounds of 6 and more spill: 192^3 485 us for 3 steps without, 508 with)
+    if (A.rounds > 5) A.rounds = 0;
     J.block0 = 0;
     J.nblocks = (J.nlines + J.lines_per_block - 1) / J.lines_per_block;
+    if (chained && h->prec == PREC_FP32) smem = line4_smem_alone(J.nblocks, smem, 0);
     CU(launch_line4_3d(h->prec, h->field_fp16, A, J.nblocks, nthreads, smem, h->stream));
     return ANISO_OK;
 }

@@ -422,7 +422,10 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     int nthreads;
     size_t smem;
     const bool ragged = v4 && (n % h->vec() != 0 || n < 2 * h->vec() || !aligned16(in) || !aligned16(out));
-    const int seg = v4 && h->seg_chunks == 0 && h->prec == PREC_FP64 ? line4_seg_fp64(n, nlines) : h->seg_chunks;
+    const int seg = !v4 || h->seg_chunks != 0   ? h->seg_chunks
+                    : h->prec == PREC_FP64 ? line4_seg_fp64(n, nlines)
+                    : ragged               ? line4_seg_ragged(nlines)
+                                           : 0;
     const int warps = v4 && transposed && h->l4_warps == 0 && h->seg_chunks == 0 && h->prec == PREC_FP32
                           ? line4_warps_alone(n, nlines)
                           : h->l4_warps;
@@ -1254,10 +1257,13 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         auto ragged = [&](const Line2Job &J) {
             return J.n % vec != 0 || J.n < 2 * vec || !aligned16(J.Tin) || !aligned16(J.Tout);
         };
+        auto seg_of = [&](const Line2Job &J) {
+            return seg == 0 && prec == PREC_FP32 && ragged(J) ? line4_seg_ragged(J.nlines) : seg;
+        };
         for (auto &J : jobs) {
             int nt;
             size_t sm;
-            if (line4_config(prec, J.n, true, warps, seg, &J.team, &J.lines_per_block, &nt, &sm, false, ragged(J)))
+            if (line4_config(prec, J.n, true, warps, seg_of(J), &J.team, &J.lines_per_block, &nt, &sm, false, ragged(J)))
                 nthreads = std::max(nthreads, nt);
         }
         // Per job: its resident blocks per SM in the shared-memory form and, when
@@ -1277,7 +1283,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             Line2Job &J = jobs[k];
             int nt = 0;
             size_t sm = 0;
-            if (!line4_config(prec, J.n, true, nthreads / 32, seg, &J.team, &J.lines_per_block, &nt, &sm, false,
+            if (!line4_config(prec, J.n, true, nthreads / 32, seg_of(J), &J.team, &J.lines_per_block, &nt, &sm, false,
                               ragged(J)) ||
                 nt != nthreads)
                 shape_rc = fail(ANISO_ERR_UNSUPPORTED, "batch: line length %d does not fit the block shape", J.n);

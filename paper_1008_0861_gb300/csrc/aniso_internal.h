@@ -215,10 +215,13 @@ int line4_blocks_per_sm(int prec, int coef_fp16, int limiter, int nthreads, size
                         int tm_cols = 64);
 // seg_chunks for an FP64 update of nlines lines of n cells launched alone.
 int line4_seg_fp64(int n, int nlines);
+// seg_chunks for an FP32 update of nlines ragged lines.
+int line4_seg_ragged(int nlines);
 // warps a block (0: the default) for an FP32 update of nlines lines of n cells launched alone.
 int line4_warps_alone(int n, int nlines);
-// dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each.
-size_t line4_smem_alone(int nblocks, size_t smem);
+// dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each (raised where that is at
+// least `from`).
+size_t line4_smem_alone(int nblocks, size_t smem, size_t from = 40 * 1024);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.
 int line4_tm_cols(int n, int team);
 // Chunks of padding after each warp's shared area in the FP32 line4 kernel

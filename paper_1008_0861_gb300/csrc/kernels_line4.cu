@@ -124,6 +124,12 @@ int line4_seg_fp64(int n, int nlines)
     return best;
 }
 
+// Chunks per lane for a ragged FP32 update (0: the default 4), alone and in
+// batches alike: short segments while every line can have a warp of its own
+// (59 x 38, two lanes of 8 chunks a line: 11.9 us an update, 8.1 on the general
+// kernel it ran on before).
+int line4_seg_ragged(int nlines) { return nlines <= 608 ? 1 : 0; }
+
 // Warps a block for one FP32 grid's update on its own.  Lines of 512 cells and
 // more (one a warp) leave a four-warp block four lines wide, so its transposed
 // store writes half sectors; eight warps write whole ones.  That is taken where
@@ -147,11 +153,13 @@ int line4_warps_alone(int n, int nlines)
 // field and step at 1024^2 45.5 / 36.9.  Short lines (under 40 KB a block) keep
 // theirs: there the SMs' switch to another split of L1 and shared memory costs
 // more (512^2, field and step 19.5 / 24.9), as does the L1 that the ragged
-// form's loads live on (1001^2 13.6 / 14.2).
-size_t line4_smem_alone(int nblocks, size_t smem)
+// form's loads live on (1001^2 13.6 / 14.2).  3-D steps, whose three launches
+// differ in their blocks, take it at any size (from = 0; 136 x 192 x 60, 3 steps
+// 201 / 141 us, 160 unchained; 100^3 127 / 132).
+size_t line4_smem_alone(int nblocks, size_t smem, size_t from)
 {
     const int share = (nblocks + 151) / 152;
-    if (share > 4 || smem < 40 * 1024) return smem;
+    if (share > 4 || smem < from) return smem;
     const size_t least = (size_t)228 * 1024 / (share + 1) - 1024 + 16;
     return smem > least ? smem : least;
 }
