@@ -8,9 +8,10 @@
 // could not write its output transposed in vectors.  Here block r of a
 // cluster holds cells [r np, (r+1) np) of four lines (12 B a cell of line
 // state), and each line's piece belongs to a team of 64 lanes (two warps,
-// 32 cells a lane at np = 2048).
+// 32 cells a lane at np = 2048); the plain state's lines up to 8192 cells go
+// eight to a block, one warp a line (32 cells a lane, np = 1024).
 //
-// The reduced system of a line (one unknown X_t per lane, 64 CS of them) is
+// The reduced system of a line (one unknown X_t per lane of its teams) is
 // solved in two levels:
 //  - within each warp, the 31 unknowns of lanes 0..30 are expressed through
 //    the two interface unknowns around them, b_{g-1} (lane 31 of the warp
@@ -18,8 +19,8 @@
 //    warp):  X_t = p_t + q_t b_{g-1} + w_t b_g, by PCR over the warp's lanes
 //    with three right-hand sides (warp shuffles, no barrier);
 //  - lane 31's own equation, with those expressions substituted, couples
-//    b_{g-1}, b_g and b_{g+1}: a cyclic tridiagonal system of G = 2 CS
-//    interface unknowns per line.  Every warp publishes the 16 numbers that
+//    b_{g-1}, b_g and b_{g+1}: a cyclic tridiagonal system of G = (warps of a
+//    team) CS interface unknowns per line.  Every warp publishes the 16 numbers that
 //    system needs in its block's shared memory; after one cluster barrier one
 //    warp per line in every block reads all G warps' numbers through
 //    distributed shared memory and solves the system by PCR over G lanes, so
