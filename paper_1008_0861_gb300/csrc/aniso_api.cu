@@ -1606,10 +1606,14 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
     }
     if (shape_rc) return shape_rc;
     // diagnostics buffers: the ring of the call and one partials region per
-    // concurrent class launch of a y-update
-    size_t part_blocks = 0;
+    // class launch of a y-update
+    // (a sweep has up to nine, three of each form, more than run side by side)
+    size_t part_blocks = 0, regions = 0;
     for (const Launch &L : launches)
-        if (L.diag_region >= 0) part_blocks = std::max(part_blocks, (size_t)L.nblocks);
+        if (L.diag_region >= 0) {
+            part_blocks = std::max(part_blocks, (size_t)L.nblocks);
+            regions = std::max(regions, (size_t)L.diag_region + 1);
+        }
     if (diag) {
         const size_t ring = (size_t)n * (size_t)max_steps * 3;
         if (ring > b->ring_count) {
@@ -1620,7 +1624,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             b->ring_count = ring;
         }
         b->ring_steps = max_steps;
-        const size_t parts = part_blocks * (1 + aniso_batch::kSide);
+        const size_t parts = part_blocks * regions;
         if (parts > b->part_count) {
             if (b->d_part) cudaFree(b->d_part);
             b->d_part = nullptr;
