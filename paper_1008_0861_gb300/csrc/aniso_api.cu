@@ -1445,6 +1445,25 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         }
     };
 
+    // A batch takes line4's block shape from its first grid's options.  Lines
+    // that do not fit it refuse the call where line4 is their only vectorised
+    // form (whole, aligned vectors; with a long FP32 side); grids that are on
+    // line4 in its ragged form, or beside long FP64 lines, then keep the general
+    // kernels, which take any line and any of the options.
+    auto on_fast_path = [&](const aniso_ctx *h, const void *Tk) {
+        if (!use_fast(h, Tk)) return false;
+        const int fk = h->fast_kind();
+        const bool whole = h->whole_vectors() && aligned16(Tk);
+        if (fk == 2 || fk == 7 || (whole && (fk == 4 || prec == PREC_FP32))) return true;
+        for (int n : {h->nx, h->ny}) {
+            int a, c, d;
+            size_t sm;
+            if (h->line4_any(n) &&
+                !line4_config(prec, n, true, b->hs[0]->l4_warps, b->hs[0]->seg_chunks, &a, &c, &d, &sm, false, true))
+                return false;
+        }
+        return true;
+    };
     size_t step_begin = 0;
     for (int s = 0; s < max_steps; ++s) {
         for (int phase = 0; phase < 2; ++phase) {
@@ -1457,7 +1476,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             for (int k = 0; k < n; ++k) {
                 if (s >= nsteps[k]) continue;
                 aniso_ctx *h = b->hs[k];
-                if (use_fast(h, T[k]) && h->fast_kind() == 7) {
+                if (on_fast_path(h, T[k]) && h->fast_kind() == 7) {
                     // cluster-kernel grids (and the compensated state): the
                     // grid's fast update captured on its own
                     Launch L{13, 0, 0, 0, 0, 0};
@@ -1468,7 +1487,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                     solo.push_back(L);
                     continue;
                 }
-                if (use_fast(h, T[k])) {
+                if (on_fast_path(h, T[k])) {
                     // x: T (rows) -> T* (column-major); y: T* (columns) -> T (rows)
                     const int per = h->bc == ANISO_BC_PERIODIC;
                     const double mu = h->chi_par * dt[k] / (h->dx * h->dy);

@@ -4,7 +4,7 @@ import numpy as np
 import pytest
 
 import workloads as W
-from gpu_util import GpuGrid
+from gpu_util import FP64_TOL_PER_STEP, GpuGrid, fp32_tol, oracle_inputs, oracle_step, rel_linf
 
 pytestmark = pytest.mark.gpu
 FP64, FP32 = 0, 1
@@ -37,3 +37,31 @@ def test_diagnostics_of_a_sweep_with_classes_of_every_form(lib):
         lib.aniso_batch_destroy(b)
         for g in grids + singles:
             g.close()
+
+
+@pytest.mark.parametrize("prec,shape,offset", [(FP32, (2001, 1501), 0), (FP32, (2000, 64), 1), (FP32, (1001, 3000), 0),
+                                               (FP64, (2000, 500), 0), (FP64, (1021, 40), 0)])
+def test_a_first_grid_with_long_segments_takes_any_other(lib, prec, shape, offset):
+    """The first grid's ANISO_OPT_SEGMENT gives the batch 16 chunks a lane,
+    which leaves long lines more than the warp-per-line kernel holds: ragged
+    grids, unaligned arrays and FP64 grids with a long side run all the same."""
+    import torch
+    first = W.random_instance(256, 128, seed=1, dt_factor=20.0)
+    inst = W.random_instance(*shape, seed=2, dt_factor=20.0)
+    a, g = GpuGrid(lib, first, prec), GpuGrid(lib, inst, prec)
+    T0, co = oracle_inputs(lib, inst, prec)
+    lib.aniso_set_option(a.h, lib.ANISO_OPT_SEGMENT, 16)
+    b = lib.aniso_batch_create([a.h, g.h])
+    try:
+        room = torch.zeros(g.T.numel() + 1, dtype=g.T.dtype, device="cuda")
+        T = room[offset:offset + g.T.numel()].view(g.T.shape)
+        T.copy_(g.T)
+        lib.aniso_step_batched(b, [a.T, T], [first.dt, inst.dt], [2, 2])
+        torch.cuda.synchronize()
+        ref = oracle_step(inst, T0, co, 2)
+        tol = 2 * FP64_TOL_PER_STEP if prec == FP64 else fp32_tol(inst, T0, co, 2, ref)
+        assert rel_linf(T.double().cpu().numpy(), ref) < tol
+    finally:
+        lib.aniso_batch_destroy(b)
+        a.close()
+        g.close()
