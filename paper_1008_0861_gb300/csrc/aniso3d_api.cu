@@ -204,7 +204,10 @@ static int enqueue3(aniso3_ctx *h, int d, const void *in, void *out, double lam,
     if (A.rounds > 5) A.rounds = 0;
     J.block0 = 0;
     J.nblocks = (J.nlines + J.lines_per_block - 1) / J.lines_per_block;
-    if (chained && h->prec == PREC_FP32) smem = line4_smem_alone(J.nblocks, smem, 0);
+    if (chained) {
+        smem = line4_smem_alone(J.nblocks, smem);
+        A.chained = line4_chain(J.nblocks, smem);
+    }
     CU(launch_line4_3d(h->prec, h->field_fp16, A, J.nblocks, nthreads, smem, h->stream));
     return ANISO_OK;
 }

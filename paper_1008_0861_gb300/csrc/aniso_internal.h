@@ -219,9 +219,10 @@ int line4_seg_fp64(int n, int nlines);
 int line4_seg_ragged(int nlines);
 // warps a block (0: the default) for an FP32 update of nlines lines of n cells launched alone.
 int line4_warps_alone(int n, int nlines);
-// dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each (raised where that is at
-// least `from`).
-size_t line4_smem_alone(int nblocks, size_t smem, size_t from = 40 * 1024);
+// dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each, and whether the launch may be
+// chained with it.
+size_t line4_smem_alone(int nblocks, size_t smem);
+bool line4_chain(int nblocks, size_t smem);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.
 int line4_tm_cols(int n, int team);
 // Chunks of padding after each warp's shared area in the FP32 line4 kernel

@@ -145,23 +145,29 @@ int line4_warps_alone(int n, int nlines)
     return blocks >= 96 && blocks <= 152 * (resident < 4 ? resident : 4) ? 8 : 0;
 }
 
-// Dynamic shared memory for a chained FP32 launch of a grid alone: enough that
-// an SM holds no more than its share of the blocks.  A chained launch's blocks
-// are placed while their predecessor drains, on whichever SMs are free first, and
-// with room for more one SM got two or three of them and another none.  us with
-// the natural size / this one: 1024^2 9.69 / 9.03 an update, 1152^2 11.5 / 10.9;
-// field and step at 1024^2 45.5 / 36.9.  Short lines (under 40 KB a block) keep
-// theirs: there the SMs' switch to another split of L1 and shared memory costs
-// more (512^2, field and step 19.5 / 24.9), as does the L1 that the ragged
-// form's loads live on (1001^2 13.6 / 14.2).  3-D steps, whose three launches
-// differ in their blocks, take it at any size (from = 0; 136 x 192 x 60, 3 steps
-// 201 / 141 us, 160 unchained; 100^3 127 / 132).
-size_t line4_smem_alone(int nblocks, size_t smem, size_t from)
+// Dynamic shared memory for a chained launch: enough that an SM holds no more
+// than its share of the blocks.  A chained launch's blocks are placed while their
+// predecessor drains, on whichever SMs are free first, and with room for more one
+// SM gets several of them and another none, which then lasts for the whole launch.
+// us, unchained / with the natural size / with this one: FP64 352 x 512, 20 steps
+// 1218 / 2762 / 1184; FP32 777 x 1001, 20 steps 533 / 754 / 518; FP32 512^2 4-step
+// 358 / 465 / 329; FP32 1024^2 an update 9.6 / 9.7 / 9.0; 3-D FP32 136 x 192 x 60,
+// 3 steps 160 / 201 / 141.
+size_t line4_smem_alone(int nblocks, size_t smem)
 {
     const int share = (nblocks + 151) / 152;
-    if (share > 4 || smem < from) return smem;
+    if (share > 4) return smem;
     const size_t least = (size_t)228 * 1024 / (share + 1) - 1024 + 16;
     return smem > least ? smem : least;
+}
+
+// Whether a launch of nblocks blocks with smem bytes each may be chained: an SM
+// has room for its share of them and no more (above), or they are so few that
+// they fit the chip beside the launch before.
+bool line4_chain(int nblocks, size_t smem)
+{
+    const int share = (nblocks + 151) / 152, room = (int)((size_t)228 * 1024 / (smem + 1024));
+    return nblocks <= 76 || room <= share;
 }
 
 // The kernel keeps 16-byte chunk c of a line at c ^ ((c >> s) & 7) inside

@@ -114,7 +114,6 @@ bool line_launch(int prec, int n, int nlines, const void *in, void *out, const v
     L->args.njobs = 1;
     L->args.limiter = LIM_VANLEER;
     L->args.err = err;
-    L->args.chained = 1;
     J.Tin = in;
     J.Tout = out;
     J.g = g;
@@ -128,7 +127,8 @@ bool line_launch(int prec, int n, int nlines, const void *in, void *out, const v
     J.swz = line4_swizzle(prec, n, J.team);
     L->args.rounds = L->ragged ? 0 : line4_rounds(prec, LIM_VANLEER, n, J.team);
     J.nblocks = (nlines + J.lines_per_block - 1) / J.lines_per_block;
-    if (prec == PREC_FP32 && !L->ragged) L->smem = line4_smem_alone(J.nblocks, L->smem);
+    L->smem = line4_smem_alone(J.nblocks, L->smem);
+    L->args.chained = line4_chain(J.nblocks, L->smem);
     return true;
 }
 
