@@ -151,10 +151,21 @@ struct aniso_ctx {
     // (line6, up to 4096 cells in whole vectors) for the others, x-then-y steps
     // only; 7: as 6, with lines the cluster kernel (line7) takes, or the
     // compensated state on line7 in both directions; 2: line2; 0: none of them.
-    int long_kernel(int n) const
+    // FP64 lines of more than 3072 cells, so few that line6's blocks (two lines
+    // each) leave half of the SMs idle, with a limiter other than van Leer (whose
+    // arithmetic line6 has not made cheaper): the general kernels, one line a
+    // block, are faster.  4 steps, us, general / line6: 4096 x 32 minmod 537 / 522,
+    // 4096 x 64 mc 669 / 704, 4096 x 128 minmod 649 / 694, 4096 x 200 mc 1366 / 1021,
+    // 3000 x 128 mc 732 / 650.
+    bool few_long_fp64(int n, int nlines) const
+    {
+        return prec == PREC_FP64 && n > 3072 && nlines >= 32 && nlines <= 152;
+    }
+    int long_kernel(int n, int nlines) const
     {
         int a, b, c;
         size_t d;
+        if (few_long_fp64(n, nlines) && limiter != LIM_VANLEER) return 0;
         if (cluster == 2 && line7_config(prec, field_fp16, n, &a, &b, &d)) return 7;
         if (line6_config(prec, field_fp16, n, &a, &b, &c, &d)) return 6;
         if (cluster != 0 && line7_config(prec, field_fp16, n, &a, &b, &d)) return 7;
@@ -188,7 +199,7 @@ struct aniso_ctx {
         if (fast == 3) {
             const bool x4 = line4_any(nx), y4 = line4_any(ny);
             if (x4 && y4) return 4;
-            const int kx = x4 ? 4 : long_kernel(nx), ky = y4 ? 4 : long_kernel(ny);
+            const int kx = x4 ? 4 : long_kernel(nx, ny), ky = y4 ? 4 : long_kernel(ny, nx);
             if (kx && ky) return (kx == 7 || ky == 7) ? 7 : 6;
         }
         if (line2_config(prec, nx, true, &a, &b, &c, &d, seg_chunks) &&
@@ -356,7 +367,9 @@ extern "C" int aniso_set_field(aniso_t h, const void *bx, const void *by)
         CU(cudaMalloc(&h->cyy, n * h->csz()));
         CU(cudaMalloc(&h->cyx, n * h->csz()));
         CU(cudaMalloc(&h->tstar, n * h->esz()));
-        if (h->col_transpose() || h->fast_shape()) {
+        // (the limiter, which can change after this, takes some shapes off the fast path)
+        if (h->col_transpose() || h->fast_shape() || h->few_long_fp64(h->nx, h->ny) ||
+            h->few_long_fp64(h->ny, h->nx)) {
             CU(cudaMalloc(&h->cyyT, n * h->csz()));
             CU(cudaMalloc(&h->cyxT, n * h->csz()));
         }
@@ -440,7 +453,7 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     // lines above line4's limit: the long-line kernels (constant diffusivity
     // only); the compensated state runs on the cluster kernel alone
     if (v4 && in_lo) ok = false;
-    const int lk = v4 && !ok && h->nl_alpha == 0.0 ? (in_lo ? 7 : h->long_kernel(n)) : 0;
+    const int lk = v4 && !ok && h->nl_alpha == 0.0 ? (in_lo ? 7 : h->long_kernel(n, nlines)) : 0;
     const bool v6 = lk == 6 && line6_config(h->prec, h->field_fp16, n, &J.team, &J.lines_per_block, &nthreads,
                                             &smem, h->l4_warps == 8 ? 2 : 4);
     int cs = 0;
