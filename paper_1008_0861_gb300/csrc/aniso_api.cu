@@ -31,16 +31,6 @@ static thread_local std::string g_last_error;
 
 extern "C" const char *aniso_last_error(void) { return g_last_error.c_str(); }
 
-bool aniso::may_chain(cudaStream_t s)
-{
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-        (void)cudaGetLastError();  // (the legacy stream while another captures: the launch itself will say)
-        return false;
-    }
-    return st == cudaStreamCaptureStatusNone;
-}
-
 // Lets other translation units of the library report through aniso_last_error.
 void aniso::record_error(const char *msg) { g_last_error = msg; }
 
@@ -105,7 +95,7 @@ struct aniso_ctx {
     int cluster = 2;    // ANISO_OPT_CLUSTER_LINES
     double nl_alpha = 0, nl_tref = 1;  // temperature-dependent diffusivity (aniso_set_nonlinear)
     // the next line kernel may be launched to overlap the end of the launch
-    // before it: one of this call's, or, outside captures, whatever it is
+    // before it: that is one of this call's
     bool chained = false;
     void *t4 = nullptr;  // intermediate of the 4-step scheme
     void *q = nullptr;   // source term (aniso_set_source), handle precision
@@ -393,7 +383,7 @@ extern "C" int aniso_set_field(aniso_t h, const void *bx, const void *by)
     }
     const double kappa = h->chi_perp / h->chi_par;
     CU(launch_face_coeffs(h->prec, h->coef_kind(), bx, by, h->nx, h->ny, h->bc, kappa, h->cxx, h->cxy,
-                          h->cyy, h->cyx, h->cyyT, h->cyxT, h->stream, may_chain(h->stream)));
+                          h->cyy, h->cyx, h->cyyT, h->cyxT, h->stream));
     h->field_set = true;
     drop_graph(h);
     return ANISO_OK;
@@ -764,7 +754,7 @@ static int enqueue_steps_any_order(aniso_ctx *h, void *T, double dt, int nsteps,
 static int enqueue_steps(aniso_ctx *h, void *T, double dt, int nsteps, long long counter0,
                          cudaStream_t s, std::vector<int> *pairs)
 {
-    h->chained = !pairs && may_chain(s);
+    h->chained = false;
     if (h->scheme == ANISO_SCHEME_EXPLICIT) {
         // explicit limited steps, T -> T* -> T ...; an odd count ends with a copy back
         ExpArgs a{};

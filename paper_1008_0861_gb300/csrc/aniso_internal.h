@@ -133,8 +133,14 @@ struct Line2Args {
     // memory (the launch's shared memory then holds two arrays, not three)
     int tmem;
     // 1: launched to start while the kernel before it in the stream drains
-    // (programmatic dependent launch); in a capture never a call's first launch
+    // (programmatic dependent launch).  Never a call's first launch: what comes
+    // before that is the caller's, perhaps itself launched so and not waiting for
+    // its own predecessor, and a chained kernel waits for the one before it alone.
     int chained;
+    // line4, chained, van Leer: 1: the kernel before writes the coefficients, which
+    // are then read with plain loads (the read-only path is for data that does not
+    // change while a kernel is resident)
+    int fresh;
     // line4, FP32 van Leer: the chunk rounds of every line of the launch, 4 to 8
     // (line4_rounds), to run the form that has them as a constant; 0: any
     int rounds;
@@ -222,6 +228,8 @@ int line4_warps_alone(int n, int nlines);
 // dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each, and whether the launch may be
 // chained with it.
 size_t line4_smem_alone(int nblocks, size_t smem);
+// whether an FP32 launch alone takes the form with three rounds of loads in flight.
+bool line4_deep(int nblocks, int nthreads);
 bool line4_chain(int nblocks, size_t smem);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.
 int line4_tm_cols(int n, int team);
@@ -266,10 +274,7 @@ cudaError_t launch_line2(int prec, int coef_fp16, const Line2Args &a, int nblock
 // the transposed copies cyyT/cyxT [nx][ny] are each optional (null).
 cudaError_t launch_face_coeffs(int bprec, int coef, const void *bx, const void *by, int nx, int ny,
                                int bc, double kappa, void *cxx, void *cxy, void *cyy, void *cyx,
-                               void *cyyT, void *cyxT, cudaStream_t s, bool chained = false);
-// Whether a call's first kernel may be launched chained: not into a capture,
-// where what comes before it may be no kernel.
-bool may_chain(cudaStream_t s);
+                               void *cyyT, void *cyxT, cudaStream_t s);
 // out[c][r] = in[r][c] for an rows x cols array of 4- or 8-byte elements.
 cudaError_t launch_transpose(int elem_bytes, const void *in, void *out, int rows, int cols,
                              cudaStream_t s);

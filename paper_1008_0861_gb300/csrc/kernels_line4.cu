@@ -19,15 +19,25 @@ template <typename K> static cudaError_t run4(K kern, const Line2Args &a, int nb
     return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
 }
 
+// A grid alone that leaves an SM at most 8 warps (of the 32 the 64-register
+// form allows) waits for its loads: three rounds in flight in the 128-register
+// form.  FP32 us an update, one round / three: 128^2 4.68 / 4.27, 512^2
+// 5.34 / 4.63, 768^2 8.21 / 7.55, 1024^2 10.4 / 10.2, 1536^2 (10 warps) 16.9 / 17.1
+bool line4_deep(int nblocks, int nthreads) { return (long)nblocks * nthreads <= 152L * 32 * 8; }
+
 cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
                          cudaStream_t s)
 {
     const bool vl = a.limiter == LIM_VANLEER;
-    // A grid alone that leaves an SM at most 16 warps (of the 32 the 64-register
-    // form allows) waits for its loads: three rounds in flight in the 128-register
-    // form.  FP32 us an update, one round / three: 128^2 4.68 / 4.27, 512^2
-    // 5.34 / 4.63, 768^2 8.21 / 7.55, 1024^2 10.4 / 10.2, 1536^2 (16 warps) 16.9 / 17.1
-    const bool deep = !a.jobs && (long)nblocks * nthreads <= 152L * 32 * 8;
+    const bool deep = !a.jobs && line4_deep(nblocks, nthreads);
+    if (a.fresh) {
+        if (!vl || a.jobs || a.one.chi_alpha != 0.0 || coef_fp16 || (prec == PREC_FP32 && !deep)) return cudaErrorInvalidValue;
+        if (prec == PREC_FP64)
+            return run4(line4_kernel<double, double, true, false, false, false, false, 1, false, 0, true>, a, nblocks,
+                        nthreads, smem, s);
+        return run4(line4_kernel<float, float, true, false, false, false, false, 3, false, 0, true>, a, nblocks,
+                    nthreads, smem, s);
+    }
     if (!a.jobs && a.one.mu == 0.0 && a.one.chi_alpha == 0.0) {  // purely implicit update (4-step halves)
         if (prec == PREC_FP64)
             return run4(line4_kernel<double, double, false, false, false, true>, a, nblocks, nthreads, smem, s);

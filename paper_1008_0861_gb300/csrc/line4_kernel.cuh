@@ -388,6 +388,7 @@ __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sy
 // constant, 0 = from the job.  The loops over rounds and segments are then
 // unrolled: no counters, and nothing moved from one chunk's registers to the
 // next's.
+// COH: the coefficients by plain loads (Line2Args::fresh; RAG's always are).
 // IMPL: a purely implicit update (no transverse term, mu = mu2 = 0: the second
 // half-update of each axis in the 4-step scheme); neighbouring lines and
 // transverse coefficients are then neither loaded nor limited.
@@ -397,7 +398,7 @@ __device__ __forceinline__ void tm_wait_st() { asm volatile("tcgen05.wait::st.sy
 // lane's chunks of T_old wait there too, from the flux phase to phase C
 // (4 V + 4 V columns of the block's 32 or 64).
 template <typename R, typename C, bool VL, bool D3 = false, bool NL = false, bool IMPL = false, bool TM = false,
-          int RING = 1, bool RAG = false, int VC = 0>
+          int RING = 1, bool RAG = false, int VC = 0, bool COH = false>
 __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4) : 2) line4_kernel(Line2Args args)
 {
     static_assert(!TM || (sizeof(R) == 4 && !D3), "TMEM line state: FP32 2-D only");
@@ -457,7 +458,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
     // (what came before is the kernel's own arguments and indices; batched
     // launches, the only ones in the tensor-memory form, are never chained)
     if (!TM && !args.jobs) chain_wait();
-    if constexpr (!TM) {  // (the kernel before may have written the coefficients)
+    if constexpr (!TM) {
         after_wait(G);
         after_wait(E);
         if constexpr (D3) after_wait(E2);
@@ -528,6 +529,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
         };
         auto ldC = [&](const C *row, int c) -> CT {
             if constexpr (RAG) return ld_ragged<N>(row, c, n, p1);
+            else if constexpr (COH) return *reinterpret_cast<const CT *>(row + c * N);
             else return ld_raw(row + c * N);
         };
         int cl[RING];

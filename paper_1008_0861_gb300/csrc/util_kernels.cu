@@ -243,20 +243,20 @@ cudaError_t launch_line2(int prec, int coef_fp16, const Line2Args &a, int nblock
 
 template <typename B, typename C>
 static cudaError_t face_launch(const void *bx, const void *by, int nx, int ny, int bc, double kappa, void *cxx,
-                               void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s, bool chained)
+                               void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s)
 {
-    return launch_kernel(face_coeffs_kernel<B, C>, dim3((nx + 31) / 32, (ny + 31) / 32), dim3(32, 8), 0, s, chained, 0,
-                         static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, kappa,
-                         static_cast<C *>(cxx), static_cast<C *>(cxy), static_cast<C *>(cyy), static_cast<C *>(cyx),
-                         static_cast<C *>(cyyT), static_cast<C *>(cyxT));
+    face_coeffs_kernel<B, C><<<dim3((nx + 31) / 32, (ny + 31) / 32), dim3(32, 8), 0, s>>>(
+        static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, kappa, static_cast<C *>(cxx),
+        static_cast<C *>(cxy), static_cast<C *>(cyy), static_cast<C *>(cyx), static_cast<C *>(cyyT),
+        static_cast<C *>(cyxT));
+    return cudaGetLastError();
 }
 
 cudaError_t launch_face_coeffs(int bprec, int coef, const void *bx, const void *by, int nx, int ny, int bc, double kappa,
-                               void *cxx, void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s,
-                               bool chained)
+                               void *cxx, void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s)
 {
     auto go = [&](auto launch) {
-        return launch(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s, chained);
+        return launch(bx, by, nx, ny, bc, kappa, cxx, cxy, cyy, cyx, cyyT, cyxT, s);
     };
     if (bprec == PREC_FP64)
         return coef == 0   ? go(face_launch<double, double>)
