@@ -798,10 +798,12 @@ __global__ void __launch_bounds__(512) col_sweep_kernel(ColArgs args)
 // From an FP64 field (or to FP64 storage) in FP64 with explicit
 // round-to-nearest operations (no contraction).  From an FP32 field to FP32 or
 // FP16 storage in double-word FP32 arithmetic (Dekker / Knuth: TwoSum, and the
-// product's error by fma), good to about 2^-46 before the one rounding: the
-// GPU does 2 FP64 operations a clock and SM, and their 18 a cell were most of
-// this kernel's time.  Components of 2^60 and more take the FP64 form (their
-// products could leave FP32's range where the coefficient does not).
+// product's error by fma): the GPU does 2 FP64 operations a clock and SM, and
+// their 18 a cell were most of this kernel's time.  The pair is within 2^-44 of
+// the value; where rounding everything within 2^-43 of it gives one stored number
+// (Ziv's test), that is what the FP64 form gives too.  Where it does not (one face
+// in 2^18), and where operations could leave FP32's range (components of 2^30 and
+// more, results under 2^-70 that are not exact zeros), the FP64 form runs.
 template <typename C> __device__ __forceinline__ C to_store(double v);
 template <> __device__ __forceinline__ double to_store<double>(double v) { return v; }
 template <> __device__ __forceinline__ float to_store<float>(double v) { return __double2float_rn(v); }
@@ -818,9 +820,23 @@ template <> __device__ __forceinline__ __half to_store2<__half>(float s, float t
     if (l != 0.f && (b & 1u) == 0u) b += ((__float_as_uint(l) ^ b) >> 31) ? ~0u : 1u;
     return __float2half_rn(__uint_as_float(b));
 }
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_uint(a) == __float_as_uint(b); }
+__device__ __forceinline__ bool same_bits(__half a, __half b) { return __half_as_ushort(a) == __half_as_ushort(b); }
+// Whether every value within 2^-43 of s + t (relative) rounds to the same C, and that C.
+template <typename C> __device__ __forceinline__ bool rounds_alike(float s, float t, C &c)
+{
+    const float d = 0x1p-43f * fabsf(s);
+    c = to_store2<C>(s, __fsub_rn(t, d));
+    return fabsf(s) >= 0x1p-70f && same_bits(c, to_store2<C>(s, __fadd_rn(t, d)));
+}
 
 struct Word2 {  // hi + lo
     float h, l;
+};
+// kappa and 1 - kappa, rounded, and as pairs.
+struct FaceConst {
+    double kappa, omk;
+    Word2 kap2, omk2;
 };
 __device__ __forceinline__ Word2 mean2(float a, float b)
 {
@@ -843,77 +859,64 @@ __device__ __forceinline__ Word2 coef2(Word2 x, Word2 y, Word2 omk, Word2 kap)
 // Both coefficients of one face: bn, bt the components along the face normal
 // and across it, in the cells before (0) and after (1) the face.
 template <typename B, typename C>
-__device__ __forceinline__ void face_coef(B bn0, B bn1, B bt0, B bt1, double kappa, C &cn, C &ct)
+__device__ __forceinline__ void face_coef(B bn0, B bn1, B bt0, B bt1, const FaceConst &fc, C &cn, C &ct)
 {
     if constexpr (sizeof(B) == 4 && sizeof(C) <= 4) {
         const float big = fmaxf(fmaxf(fabsf(bn0), fabsf(bn1)), fmaxf(fabsf(bt0), fabsf(bt1)));
-        if (big < 0x1p60f) {
-            const double o = __dsub_rn(1.0, kappa);
-            Word2 omk, kap;
-            omk.h = __double2float_rn(o);
-            omk.l = __double2float_rn(__dsub_rn(o, (double)omk.h));
-            kap.h = __double2float_rn(kappa);
-            kap.l = __double2float_rn(__dsub_rn(kappa, (double)kap.h));
-            const Word2 fn = mean2(bn0, bn1), ft = mean2(bt0, bt1);
-            const Word2 n = coef2(fn, fn, omk, kap), t = coef2(fn, ft, omk, Word2{0.f, 0.f});
-            cn = to_store2<C>(n.h, n.l);
-            ct = to_store2<C>(t.h, t.l);
-            return;
-        }
+        const Word2 fn = mean2(bn0, bn1), ft = mean2(bt0, bt1);
+        const Word2 n = coef2(fn, fn, fc.omk2, fc.kap2), t = coef2(fn, ft, fc.omk2, Word2{0.f, 0.f});
+        bool ok = big < 0x1p30f;
+        if (fn.h == 0.f) cn = to_store2<C>(fc.kap2.h, fc.kap2.l);
+        else ok = rounds_alike<C>(n.h, n.l, cn) && ok;
+        if (fn.h == 0.f || ft.h == 0.f) ct = to_store2<C>(__fmul_rn(fc.omk2.h, __fmul_rn(fn.h, ft.h)), 0.f);
+        else ok = rounds_alike<C>(t.h, t.l, ct) && ok;
+        if (ok) return;
     }
-    const double omk = __dsub_rn(1.0, kappa);
     const double fn = __dmul_rn(0.5, __dadd_rn((double)bn0, (double)bn1));
     const double ft = __dmul_rn(0.5, __dadd_rn((double)bt0, (double)bt1));
-    cn = to_store<C>(__dadd_rn(kappa, __dmul_rn(omk, __dmul_rn(fn, fn))));
-    ct = to_store<C>(__dmul_rn(omk, __dmul_rn(fn, ft)));
+    cn = to_store<C>(__dadd_rn(fc.kappa, __dmul_rn(fc.omk, __dmul_rn(fn, fn))));
+    ct = to_store<C>(__dmul_rn(fc.omk, __dmul_rn(fn, ft)));
 }
 
-// One block a 32 x 32 tile of cells (32 x 8 threads).  The y faces' values go
+// One block a tile of 32 x 8 cells, one thread a cell.  The y faces' values go
 // out in the natural layout (cyy, cyx) and, where asked for (cyyT, cyxT),
-// through shared memory as whole rows of the transposed one: written by
+// through shared memory as pieces of 8 cells of the transposed one: written by
 // column from the natural order, every 4-byte store was a sector of its own.
-// 1024^2 FP32: 64 us a call with both, 8 now.
+// us a call with both, by columns / tiles of 32 x 32 cells on 256 threads / this:
+// FP32 1024^2 64.0 / 14.6 / 12.8, 64^2 4.6 / 6.6 / 3.5; FP64 1024^2 42.9 / 42.8 /
+// 39.6, 64^2 4.4 / 9.6 / 4.6 (larger tiles crowd a small grid's FP64 work on few SMs).
 template <typename B, typename C>
-__global__ void __launch_bounds__(256) face_coeffs_kernel(const B *bx, const B *by, int nx,
-                                                          int ny, int bc, double kappa, C *cxx, C *cxy, C *cyy, C *cyx,
-                                                          C *cyyT, C *cyxT)
+__global__ void __launch_bounds__(256) face_coeffs_kernel(const B *bx, const B *by, int nx, int ny, int bc, FaceConst fc,
+                                                          C *cxx, C *cxy, C *cyy, C *cyx, C *cyyT, C *cyxT)
 {
-    __shared__ C tyy[32][33], tyx[32][33];
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32;
-    const int i = i0 + threadIdx.x;
+    __shared__ C tyy[8][33], tyx[8][33];
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 8;
+    const int i = i0 + threadIdx.x, j = j0 + threadIdx.y;
     const bool per = bc == 1;  // otherwise the boundary faces carry no flux
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int r = threadIdx.y + 8 * k, j = j0 + r;
-        if (i < nx && j < ny) {
-            const size_t o = (size_t)j * nx + i;
-            const size_t ox = i + 1 < nx ? o + 1 : o - (nx - 1);
-            const size_t oy = j + 1 < ny ? o + nx : (size_t)i;
-            const B x0 = __ldg(bx + o), y0 = __ldg(by + o);
-            C vxx = C(0.f), vxy = C(0.f), vyy = C(0.f), vyx = C(0.f);
-            if (per || i != nx - 1) face_coef<B, C>(x0, __ldg(bx + ox), y0, __ldg(by + ox), kappa, vxx, vxy);
-            if (per || j != ny - 1) face_coef<B, C>(y0, __ldg(by + oy), x0, __ldg(bx + oy), kappa, vyy, vyx);
-            cxx[o] = vxx;
-            cxy[o] = vxy;
-            if (cyy) {
-                cyy[o] = vyy;
-                cyx[o] = vyx;
-            }
-            tyy[r][threadIdx.x] = vyy;
-            tyx[r][threadIdx.x] = vyx;
+    if (i < nx && j < ny) {
+        const size_t o = (size_t)j * nx + i;
+        const size_t ox = i + 1 < nx ? o + 1 : o - (nx - 1);
+        const size_t oy = j + 1 < ny ? o + nx : (size_t)i;
+        const B x0 = __ldg(bx + o), y0 = __ldg(by + o);
+        C vxx = C(0.f), vxy = C(0.f), vyy = C(0.f), vyx = C(0.f);
+        if (per || i != nx - 1) face_coef<B, C>(x0, __ldg(bx + ox), y0, __ldg(by + ox), fc, vxx, vxy);
+        if (per || j != ny - 1) face_coef<B, C>(y0, __ldg(by + oy), x0, __ldg(bx + oy), fc, vyy, vyx);
+        cxx[o] = vxx;
+        cxy[o] = vxy;
+        if (cyy) {
+            cyy[o] = vyy;
+            cyx[o] = vyx;
         }
+        tyy[threadIdx.y][threadIdx.x] = vyy;
+        tyx[threadIdx.y][threadIdx.x] = vyx;
     }
     if (!cyyT) return;
     __syncthreads();
-    const int j = j0 + threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int c = threadIdx.y + 8 * k;
-        if (i0 + c < nx && j < ny) {
-            const size_t oT = (size_t)(i0 + c) * ny + j;
-            cyyT[oT] = tyy[threadIdx.x][c];
-            cyxT[oT] = tyx[threadIdx.x][c];
-        }
+    const int e = threadIdx.y * 32 + threadIdx.x, r = e & 7, c = e >> 3;
+    if (i0 + c < nx && j0 + r < ny) {
+        const size_t oT = (size_t)(i0 + c) * ny + j0 + r;
+        cyyT[oT] = tyy[r][c];
+        cyxT[oT] = tyx[r][c];
     }
 }
 

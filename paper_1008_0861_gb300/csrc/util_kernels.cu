@@ -245,8 +245,11 @@ template <typename B, typename C>
 static cudaError_t face_launch(const void *bx, const void *by, int nx, int ny, int bc, double kappa, void *cxx,
                                void *cxy, void *cyy, void *cyx, void *cyyT, void *cyxT, cudaStream_t s)
 {
-    face_coeffs_kernel<B, C><<<dim3((nx + 31) / 32, (ny + 31) / 32), dim3(32, 8), 0, s>>>(
-        static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, kappa, static_cast<C *>(cxx),
+    auto pair = [](double v) { return Word2{(float)v, (float)(v - (double)(float)v)}; };
+    const double omk = 1.0 - kappa;
+    const FaceConst fc{kappa, omk, pair(kappa), pair(omk)};
+    face_coeffs_kernel<B, C><<<dim3((nx + 31) / 32, (ny + 7) / 8), dim3(32, 8), 0, s>>>(
+        static_cast<const B *>(bx), static_cast<const B *>(by), nx, ny, bc, fc, static_cast<C *>(cxx),
         static_cast<C *>(cxy), static_cast<C *>(cyy), static_cast<C *>(cyx), static_cast<C *>(cyyT),
         static_cast<C *>(cyxT));
     return cudaGetLastError();
