@@ -868,7 +868,7 @@ __device__ __forceinline__ void face_coef(B bn0, B bn1, B bt0, B bt1, const Face
         bool ok = big < 0x1p30f;
         if (fn.h == 0.f) cn = to_store2<C>(fc.kap2.h, fc.kap2.l);
         else ok = rounds_alike<C>(n.h, n.l, cn) && ok;
-        if (fn.h == 0.f || ft.h == 0.f) ct = to_store2<C>(__fmul_rn(fc.omk2.h, __fmul_rn(fn.h, ft.h)), 0.f);
+        if (fn.h == 0.f || ft.h == 0.f) ct = C(__fmul_rn(fc.omk2.h, __fmul_rn(fn.h, ft.h)));  // 0, of the products' sign
         else ok = rounds_alike<C>(t.h, t.l, ct) && ok;
         if (ok) return;
     }
