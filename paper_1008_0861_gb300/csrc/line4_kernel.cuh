@@ -112,8 +112,8 @@ template <> struct Fast<float> {
 // and SM), and divisions were most of its 98 a cell.  1/x here is one
 // third-order Newton step (Chebyshev's method) from the hardware's 20-bit
 // estimate: with e = 1 - x y, y (1 + e + e^2) = (1 - e^3) / x, three fused
-// operations, within 1 ulp.  x must be normal; an estimate that underflows
-// gives 0, an infinite x NaN.
+// operations, within 1 ulp.  x and 1/x must be normal: |x| from 2^-1022 to 2^1022
+// (an estimate that underflows gives 0, an infinite x NaN).
 __device__ __forceinline__ double drcp_approx(double x)
 {
     double y;
@@ -121,9 +121,13 @@ __device__ __forceinline__ double drcp_approx(double x)
     const double e = __fma_rn(-x, y, 1.0);
     return __fma_rn(y, __fma_rn(e, e, e), y);
 }
-// Correctly rounded quotient and reciprocal from such a y: one step with the
-// exact remainder (Markstein, IBM J. Res. Dev. 34, 1990), the same bits as an
-// IEEE division wherever remainder and quotient are normal numbers.
+// Quotient and reciprocal from such a y by one step with the exact remainder
+// (Markstein, IBM J. Res. Dev. 34, 1990).  y is not the rounded 1/b that his proof
+// of correct rounding asks for, but within 1 ulp of it, and the value before the
+// last rounding within 2^-51 ulp of the quotient: the result is the rounded one
+// unless the quotient lies that close to the middle of two numbers (1/x of an
+// x = 2^k (2 - 2^-52) does), and the other neighbour then.  Quotient and
+// remainder must be normal numbers.
 __device__ __forceinline__ double dquot(double a, double b, double y)
 {
     const double q = a * y;
