@@ -173,40 +173,74 @@ template <typename R, bool VL, bool HARMONIC = false> struct Limit {
     static __device__ __forceinline__ R inner(int lim, R a, R b) { return level<R, VL>(lim, a, b); }
     static __device__ __forceinline__ R outer(int lim, R v, R w) { return level<R, VL>(lim, v, w); }
 };
-// FP64 van Leer, the nest as written: a cell keeps ab / (a + b), half of its
-// level, a face forms the same quotient of two cells', a quarter of the nest
-// (powers of two: the bits of the nest of 2ab / (a + b)).  Signs and zeros are
-// told from the high words, off the FP64 pipe; products below the smallest
-// normal number (differences under 1e-154) and non-finite ones give 0.
-// A run amplifies the last bit (the ring at 1000 times the limit by 1e6 in a
-// hundred steps), which is why the quotients keep their rounding.
+// FP64 van Leer.  A product in [2^-960, 2^1020) leaves quotient and remainder
+// normal; others are told from the high word, off the FP64 pipe.
+__device__ __forceinline__ bool vl_plain(double p) { return (unsigned)(__double2hiint(p) - 0x03f00000) < 0x7bc00000u; }
+// Neither factor of a product p outside that range is 0, and p is not negative.
+__device__ __forceinline__ bool vl_edge_of(double p, double a, double b)
+{
+    const int za = (__double2hiint(a) << 1) | __double2loint(a), zb = (__double2hiint(b) << 1) | __double2loint(b);
+    return __double2hiint(p) >= 0 && za != 0 && zb != 0;
+}
+// Half of a level for such a product: as lim2 forms it.
+static __device__ __noinline__ double vl_edge(double a, double b)
+{
+    return 0.5 * lim2<double>(LIM_VANLEER, a, b);
+}
+// The nest as written: a cell keeps ab / (a + b), half of its level, a face
+// forms the same quotient of two cells', a quarter of the nest (powers of two:
+// the bits of the nest of 2ab / (a + b)).  A run amplifies the last bit (the ring
+// at 1000 times the limit by 1e6 in a hundred steps), which is why the quotients
+// keep their rounding.
 template <> struct Limit<double, true, false> {
     static constexpr int SCALE = 4;
     static __device__ __forceinline__ double inner(int, double a, double b)
     {
         const double p = a * b, s = a + b;
         const double q = dquot(p, s, drcp_approx(s));
-        return (unsigned)(__double2hiint(p) - 0x00100000) < 0x7fe00000u ? q : 0.0;
+        if (vl_plain(p)) return q;
+        return vl_edge_of(p, a, b) ? vl_edge(a, b) : 0.0;
     }
-    static __device__ __forceinline__ double outer(int lim, double v, double w) { return inner(lim, v, w); }
+    static __device__ __forceinline__ double outer(int, double v, double w)
+    {
+        const double p = v * w, s = v + w;
+        const double q = dquot(p, s, drcp_approx(s));
+        if (vl_plain(p)) return q;
+        return vl_edge_of(p, v, w) ? 0.5 * vl_edge(2.0 * v, 2.0 * w) : 0.0;
+    }
 };
-// FP64 van Leer by sums of reciprocals (the long lines, whose segments are
-// others than they were): L is the harmonic mean, so the nest is
-// 4 / (1/a + 1/b + 1/c + 1/d) where all four share a sign.  A cell keeps
-// w = 1/a + 1/b = (a + b) / (a b) (0 where the signs differ), a face takes
-// 1 / (w_p + w_{p+1}): 12 operations a cell instead of 18, the same range.
+// By sums of reciprocals (the long lines, whose segments are others than they
+// were): L is the harmonic mean, so the nest is 4 / (1/a + 1/b + 1/c + 1/d)
+// where all four share a sign.  A cell keeps w = 1/a + 1/b = (a + b) / (a b) (0
+// where the signs differ or the level is next to 0, NaN where it leaves the
+// range), a face takes 1 / (w_p + w_{p+1}): 12 operations a cell instead of 18.
 template <> struct Limit<double, true, true> {
     static constexpr int SCALE = 4;
+    static __device__ __noinline__ double edge(double a, double b)
+    {
+        const double h = vl_edge(a, b), m = fabs(h);
+        if (m < 0x1p-1000) return 0.0;
+        return m < INFINITY ? 1.0 / h : copysign(__longlong_as_double(0x7ff8000000000000ll), a);
+    }
     static __device__ __forceinline__ double inner(int, double a, double b)
     {
         const double p = a * b, w = (a + b) * drcp_approx(p);
-        return (unsigned)(__double2hiint(p) - 0x00100000) < 0x7fe00000u ? w : 0.0;
+        if (vl_plain(p)) return w;
+        return vl_edge_of(p, a, b) ? edge(a, b) : 0.0;
+    }
+    // (2 / v and 2 / w are the cells' levels)
+    static __device__ __noinline__ double outer_edge(double v, double w)
+    {
+        return fabs(v + w) < INFINITY ? 0.25 * lim2<double>(LIM_VANLEER, 2.0 / v, 2.0 / w) : v + w;
     }
     static __device__ __forceinline__ double outer(int, double v, double w)
     {
         const int hv = __double2hiint(v), hw = __double2hiint(w);
         const double r = drcp_approx(v + w);
-        return hv != 0 && hw != 0 && (hv ^ hw) >= 0 ? r : 0.0;
+        if (hv == 0 || hw == 0 || (hv ^ hw) < 0) return 0.0;
+        // levels whose product is under 2^-950 (or NaN): as lim2 rounds it
+        const unsigned e = (unsigned)(hv & 0x7fffffff) + (unsigned)(hw & 0x7fffffff);
+        return e < 0xbba00000u ? r : outer_edge(v, w);
     }
 };
 
