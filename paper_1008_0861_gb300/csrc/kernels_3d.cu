@@ -89,21 +89,6 @@ cudaError_t launch_face_coeffs3(int prec, int coef_fp16, const void *bx, const v
     return cudaGetLastError();
 }
 
-template <typename K> static cudaError_t run4_3d(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem,
-                                                 cudaStream_t s)
-{
-    if (smem > 47 * 1024) {  // static shared memory counts against the 48 KB default
-        cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-        if (e != cudaSuccess) return e;
-        if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-                cudaSuccess)
-            return e;
-    }
-    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
-}
-
 cudaError_t launch_line4_3d(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
                             cudaStream_t s)
 {
@@ -111,20 +96,20 @@ cudaError_t launch_line4_3d(int prec, int coef_fp16, const Line2Args &a, int nbl
     if (coef_fp16 && prec == PREC_FP64) return cudaErrorInvalidValue;
     if (a.one.mu == 0.0 && a.one.mu2 == 0.0) {  // purely implicit update (4-step halves)
         if (prec == PREC_FP64)
-            return run4_3d(line4_kernel<double, double, false, true, false, true>, a, nblocks, nthreads, smem, s);
+            return launch_line_kernel(line4_kernel<double, double, false, true, false, true>, a, nblocks, nthreads, smem, s);
         if (coef_fp16)
-            return run4_3d(line4_kernel<float, __half, false, true, false, true>, a, nblocks, nthreads, smem, s);
-        return run4_3d(line4_kernel<float, float, false, true, false, true>, a, nblocks, nthreads, smem, s);
+            return launch_line_kernel(line4_kernel<float, __half, false, true, false, true>, a, nblocks, nthreads, smem, s);
+        return launch_line_kernel(line4_kernel<float, float, false, true, false, true>, a, nblocks, nthreads, smem, s);
     }
     if (prec == PREC_FP32 && a.rounds) return launch_line4_rounds_3d(coef_fp16, a, nblocks, nthreads, smem, s);
     if (coef_fp16)
-        return vl ? run4_3d(line4_kernel<float, __half, true, true>, a, nblocks, nthreads, smem, s)
-                  : run4_3d(line4_kernel<float, __half, false, true>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line4_kernel<float, __half, true, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line4_kernel<float, __half, false, true>, a, nblocks, nthreads, smem, s);
     if (prec == PREC_FP64)
-        return vl ? run4_3d(line4_kernel<double, double, true, true>, a, nblocks, nthreads, smem, s)
-                  : run4_3d(line4_kernel<double, double, false, true>, a, nblocks, nthreads, smem, s);
-    return vl ? run4_3d(line4_kernel<float, float, true, true>, a, nblocks, nthreads, smem, s)
-              : run4_3d(line4_kernel<float, float, false, true>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line4_kernel<double, double, true, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line4_kernel<double, double, false, true>, a, nblocks, nthreads, smem, s);
+    return vl ? launch_line_kernel(line4_kernel<float, float, true, true>, a, nblocks, nthreads, smem, s)
+              : launch_line_kernel(line4_kernel<float, float, false, true>, a, nblocks, nthreads, smem, s);
 }
 
 }  // namespace aniso

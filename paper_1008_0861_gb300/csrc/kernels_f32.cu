@@ -3,23 +3,10 @@
 
 namespace aniso {
 
-// Opt in to the dynamic shared memory a launch needs (above the 48 KB
-// default), never more than requested so the kernel's static shared memory
-// still fits under the per-block limit.
-template <typename K> static cudaError_t prep(K kern, size_t smem)
-{
-    if (smem <= 47 * 1024) return cudaSuccess;  // static shared memory counts too
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess) return e;
-    if ((size_t)fa.maxDynamicSharedSizeBytes >= smem) return cudaSuccess;
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 template <typename K> static cudaError_t go(K kern, int nblocks, int nthreads, size_t smem, cudaStream_t s,
                                               const LineArgs &a)
 {
-    cudaError_t err = prep(kern, smem);
+    cudaError_t err = allow_smem(kern, smem);
     if (err != cudaSuccess) return err;
     kern<<<nblocks, nthreads, smem, s>>>(a);
     return cudaGetLastError();
@@ -27,7 +14,7 @@ template <typename K> static cudaError_t go(K kern, int nblocks, int nthreads, s
 template <typename K> static cudaError_t goc(K kern, int nblocks, int nthreads, size_t smem, cudaStream_t s,
                                                const ColArgs &a)
 {
-    cudaError_t err = prep(kern, smem);
+    cudaError_t err = allow_smem(kern, smem);
     if (err != cudaSuccess) return err;
     kern<<<nblocks, nthreads, smem, s>>>(a);
     return cudaGetLastError();
@@ -56,7 +43,7 @@ cudaError_t launch_col_f32(int coef_fp16, bool kahan, const ColArgs &a, int nblo
 template <typename K> static cudaError_t go2(K kern, int nblocks, int nthreads, size_t smem, cudaStream_t s,
                                                const Line2Args &a)
 {
-    cudaError_t err = prep(kern, smem);
+    cudaError_t err = allow_smem(kern, smem);
     if (err != cudaSuccess) return err;
     kern<<<nblocks, nthreads, smem, s>>>(a);
     return cudaGetLastError();

@@ -4,21 +4,6 @@
 
 namespace aniso {
 
-template <typename K> static cudaError_t run4(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem,
-                                              cudaStream_t s)
-{
-    if (smem > 47 * 1024) {  // static shared memory counts against the 48 KB default
-        cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-        if (e != cudaSuccess) return e;
-        if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-                cudaSuccess)
-            return e;
-    }
-    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
-}
-
 // A grid alone that leaves an SM at most 8 warps (of the 32 the 64-register
 // form allows) waits for its loads: three rounds in flight in the 128-register
 // form.  FP32 us an update, one round / three: 128^2 4.68 / 4.27, 512^2
@@ -33,61 +18,55 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
     if (a.fresh) {
         if (!vl || a.jobs || a.one.chi_alpha != 0.0 || coef_fp16 || (prec == PREC_FP32 && !deep)) return cudaErrorInvalidValue;
         if (prec == PREC_FP64)
-            return run4(line4_kernel<double, double, true, false, false, false, false, 1, false, 0, true>, a, nblocks,
+            return launch_line_kernel(line4_kernel<double, double, true, false, false, false, false, 1, false, 0, true>, a, nblocks,
                         nthreads, smem, s);
-        return run4(line4_kernel<float, float, true, false, false, false, false, 3, false, 0, true>, a, nblocks,
+        return launch_line_kernel(line4_kernel<float, float, true, false, false, false, false, 3, false, 0, true>, a, nblocks,
                     nthreads, smem, s);
     }
     if (!a.jobs && a.one.mu == 0.0 && a.one.chi_alpha == 0.0) {  // purely implicit update (4-step halves)
         if (prec == PREC_FP64)
-            return run4(line4_kernel<double, double, false, false, false, true>, a, nblocks, nthreads, smem, s);
+            return launch_line_kernel(line4_kernel<double, double, false, false, false, true>, a, nblocks, nthreads, smem, s);
         if (coef_fp16)
-            return run4(line4_kernel<float, __half, false, false, false, true>, a, nblocks, nthreads, smem, s);
-        return run4(line4_kernel<float, float, false, false, false, true>, a, nblocks, nthreads, smem, s);
+            return launch_line_kernel(line4_kernel<float, __half, false, false, false, true>, a, nblocks, nthreads, smem, s);
+        return launch_line_kernel(line4_kernel<float, float, false, false, false, true>, a, nblocks, nthreads, smem, s);
     }
     if (!a.jobs && a.one.chi_alpha != 0.0) {  // temperature-dependent diffusivity (single grids)
         if (coef_fp16) return cudaErrorInvalidValue;
         if (prec == PREC_FP64)
-            return vl ? run4(line4_kernel<double, double, true, false, true>, a, nblocks, nthreads, smem, s)
-                      : run4(line4_kernel<double, double, false, false, true>, a, nblocks, nthreads, smem, s);
+            return vl ? launch_line_kernel(line4_kernel<double, double, true, false, true>, a, nblocks, nthreads, smem, s)
+                      : launch_line_kernel(line4_kernel<double, double, false, false, true>, a, nblocks, nthreads, smem, s);
         if (vl && deep && a.rounds) return launch_line4_rounds(0, true, a, nblocks, nthreads, smem, s);
         if (vl && deep)
-            return run4(line4_kernel<float, float, true, false, true, false, false, 3>, a, nblocks, nthreads, smem, s);
-        return vl ? run4(line4_kernel<float, float, true, false, true>, a, nblocks, nthreads, smem, s)
-                  : run4(line4_kernel<float, float, false, false, true>, a, nblocks, nthreads, smem, s);
+            return launch_line_kernel(line4_kernel<float, float, true, false, true, false, false, 3>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line4_kernel<float, float, true, false, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line4_kernel<float, float, false, false, true>, a, nblocks, nthreads, smem, s);
     }
     if (a.tmem && prec == PREC_FP32) {  // gamma in tensor memory
         if (a.rounds) return launch_line4_rounds_tm(coef_fp16, a, nblocks, nthreads, smem, s);
         if (coef_fp16)
-            return vl ? run4(line4_kernel<float, __half, true, false, false, false, true>, a, nblocks, nthreads, smem, s)
-                      : run4(line4_kernel<float, __half, false, false, false, false, true>, a, nblocks, nthreads, smem, s);
-        return vl ? run4(line4_kernel<float, float, true, false, false, false, true>, a, nblocks, nthreads, smem, s)
-                  : run4(line4_kernel<float, float, false, false, false, false, true>, a, nblocks, nthreads, smem, s);
+            return vl ? launch_line_kernel(line4_kernel<float, __half, true, false, false, false, true>, a, nblocks, nthreads, smem, s)
+                      : launch_line_kernel(line4_kernel<float, __half, false, false, false, false, true>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line4_kernel<float, float, true, false, false, false, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line4_kernel<float, float, false, false, false, false, true>, a, nblocks, nthreads, smem, s);
     }
     if (prec == PREC_FP64)
-        return vl ? run4(line4_kernel<double, double, true>, a, nblocks, nthreads, smem, s)
-                  : run4(line4_kernel<double, double, false>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line4_kernel<double, double, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line4_kernel<double, double, false>, a, nblocks, nthreads, smem, s);
     if (prec == PREC_FP32 && a.rounds) return launch_line4_rounds(coef_fp16, deep, a, nblocks, nthreads, smem, s);
     if (vl && deep)
-        return coef_fp16 ? run4(line4_kernel<float, __half, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s)
-                         : run4(line4_kernel<float, float, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s);
+        return coef_fp16 ? launch_line_kernel(line4_kernel<float, __half, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s)
+                         : launch_line_kernel(line4_kernel<float, float, true, false, false, false, false, 3>, a, nblocks, nthreads, smem, s);
     if (coef_fp16)
-        return vl ? run4(line4_kernel<float, __half, true>, a, nblocks, nthreads, smem, s)
-                  : run4(line4_kernel<float, __half, false>, a, nblocks, nthreads, smem, s);
-    return vl ? run4(line4_kernel<float, float, true>, a, nblocks, nthreads, smem, s)
-              : run4(line4_kernel<float, float, false>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line4_kernel<float, __half, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line4_kernel<float, __half, false>, a, nblocks, nthreads, smem, s);
+    return vl ? launch_line_kernel(line4_kernel<float, float, true>, a, nblocks, nthreads, smem, s)
+              : launch_line_kernel(line4_kernel<float, float, false>, a, nblocks, nthreads, smem, s);
 }
 
 template <typename K> static int occ4(K kern, int nthreads, size_t smem)
 {
-    if (smem > 47 * 1024) {
-        cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return -1;
-        if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return -1;
-    }
     int blocks = 0;
+    if (allow_smem(kern, smem) != cudaSuccess) return -1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kern, nthreads, smem) != cudaSuccess) return -1;
     return blocks;
 }

@@ -8,9 +8,9 @@ namespace aniso {
 template <int VC> struct Cube {
     static cudaError_t run(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
     {
-        return coef_fp16 ? run_rounds(line4_kernel<float, __half, true, true, false, false, false, 1, false, VC>, a,
+        return coef_fp16 ? launch_line_kernel(line4_kernel<float, __half, true, true, false, false, false, 1, false, VC>, a,
                                       nblocks, nthreads, smem, s)
-                         : run_rounds(line4_kernel<float, float, true, true, false, false, false, 1, false, VC>, a,
+                         : launch_line_kernel(line4_kernel<float, float, true, true, false, false, false, 1, false, VC>, a,
                                       nblocks, nthreads, smem, s);
     }
 };

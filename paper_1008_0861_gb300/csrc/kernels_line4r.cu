@@ -8,15 +8,6 @@ template <typename R, typename C, bool VL, int RING>
 static cudaError_t run4r(const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
 {
     auto kern = line4_kernel<R, C, VL, false, false, false, false, RING, true>;
-    if (smem > 47 * 1024) {  // static shared memory counts against the 48 KB default
-        cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-        if (e != cudaSuccess) return e;
-        if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-                cudaSuccess)
-            return e;
-    }
     return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
 }
 

@@ -7,9 +7,9 @@ namespace aniso {
 template <int VC> struct Tensor {
     static cudaError_t run(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
     {
-        return coef_fp16 ? run_rounds(line4_kernel<float, __half, true, false, false, false, true, 1, false, VC>, a,
+        return coef_fp16 ? launch_line_kernel(line4_kernel<float, __half, true, false, false, false, true, 1, false, VC>, a,
                                       nblocks, nthreads, smem, s)
-                         : run_rounds(line4_kernel<float, float, true, false, false, false, true, 1, false, VC>, a,
+                         : launch_line_kernel(line4_kernel<float, float, true, false, false, false, true, 1, false, VC>, a,
                                       nblocks, nthreads, smem, s);
     }
 };

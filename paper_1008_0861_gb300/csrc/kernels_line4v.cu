@@ -11,9 +11,9 @@ namespace aniso {
 template <int VC> struct Plain {
     static cudaError_t run(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
     {
-        return coef_fp16 ? run_rounds(line4_kernel<float, __half, true, false, false, false, false, 1, false, VC>, a,
+        return coef_fp16 ? launch_line_kernel(line4_kernel<float, __half, true, false, false, false, false, 1, false, VC>, a,
                                       nblocks, nthreads, smem, s)
-                         : run_rounds(line4_kernel<float, float, true, false, false, false, false, 1, false, VC>, a,
+                         : launch_line_kernel(line4_kernel<float, float, true, false, false, false, false, 1, false, VC>, a,
                                       nblocks, nthreads, smem, s);
     }
 };
@@ -21,11 +21,11 @@ template <int VC> struct Alone {
     static cudaError_t run(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
     {
         if (a.one.chi_alpha != 0.0)
-            return run_rounds(line4_kernel<float, float, true, false, true, false, false, 3, false, VC>, a, nblocks,
+            return launch_line_kernel(line4_kernel<float, float, true, false, true, false, false, 3, false, VC>, a, nblocks,
                               nthreads, smem, s);
-        return coef_fp16 ? run_rounds(line4_kernel<float, __half, true, false, false, false, false, 3, false, VC>, a,
+        return coef_fp16 ? launch_line_kernel(line4_kernel<float, __half, true, false, false, false, false, 3, false, VC>, a,
                                       nblocks, nthreads, smem, s)
-                         : run_rounds(line4_kernel<float, float, true, false, false, false, false, 3, false, VC>, a,
+                         : launch_line_kernel(line4_kernel<float, float, true, false, false, false, false, 3, false, VC>, a,
                                       nblocks, nthreads, smem, s);
     }
 };

@@ -52,11 +52,7 @@ template <bool VL> void *kernel_ptr() { return reinterpret_cast<void *>(line5_ke
 
 int grid_limit(const void *kern, int nthreads, size_t smem)
 {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return -1;
-    if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return -1;
+    if (allow_smem(kern, smem) != cudaSuccess) return -1;
     int per_sm = 0, dev = 0, sms = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nthreads, smem) != cudaSuccess) return -1;
     if (cudaGetDevice(&dev) != cudaSuccess ||

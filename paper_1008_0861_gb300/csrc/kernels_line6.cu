@@ -30,29 +30,17 @@ bool line6_config(int prec, int coef_fp16, int n, int *team, int *lines_per_bloc
     return true;
 }
 
-template <typename K> static cudaError_t run6(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem,
-                                              cudaStream_t s)
-{
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess) return e;
-    if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-        (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
-    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
-}
-
 cudaError_t launch_line6(int prec, int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
 {
     const bool vl = a.limiter == LIM_VANLEER;
     if (prec == PREC_FP64)
-        return vl ? run6(line6_kernel<double, double, true>, a, nblocks, nthreads, smem, s)
-                  : run6(line6_kernel<double, double, false>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line6_kernel<double, double, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line6_kernel<double, double, false>, a, nblocks, nthreads, smem, s);
     if (coef_fp16)
-        return vl ? run6(line6_kernel<float, __half, true>, a, nblocks, nthreads, smem, s)
-                  : run6(line6_kernel<float, __half, false>, a, nblocks, nthreads, smem, s);
-    return vl ? run6(line6_kernel<float, float, true>, a, nblocks, nthreads, smem, s)
-              : run6(line6_kernel<float, float, false>, a, nblocks, nthreads, smem, s);
+        return vl ? launch_line_kernel(line6_kernel<float, __half, true>, a, nblocks, nthreads, smem, s)
+                  : launch_line_kernel(line6_kernel<float, __half, false>, a, nblocks, nthreads, smem, s);
+    return vl ? launch_line_kernel(line6_kernel<float, float, true>, a, nblocks, nthreads, smem, s)
+              : launch_line_kernel(line6_kernel<float, float, false>, a, nblocks, nthreads, smem, s);
 }
 
 }  // namespace aniso

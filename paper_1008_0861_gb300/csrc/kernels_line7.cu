@@ -33,12 +33,6 @@ bool line7_config(int prec, int coef_fp16, int n, int *cs, int *nthreads, size_t
 template <typename Kern>
 static cudaError_t run7(Kern kern, const Line2Args &a, int lines, int cs, size_t smem, cudaStream_t s)
 {
-    cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-    if (e != cudaSuccess) return e;
-    if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-        (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
     const int groups = (a.one.nlines + lines - 1) / lines;
     // (never chained: launches of 100 us and more gain nothing, 4096^2 lost 0.4 %)
     return launch_line_kernel(kern, a, groups * cs, L7_THREADS, smem, s, cs);

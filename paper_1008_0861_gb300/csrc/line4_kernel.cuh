@@ -89,11 +89,13 @@ __device__ __forceinline__ void l2_prefetch(const void *p, size_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"((unsigned)bytes) : "memory");
 }
 
-// Host: a launch of kern(a) in a.chained mode or plainly.
+// Host: a launch of kern(a) in a.chained mode or plainly, with any amount of shared memory.
 template <typename K>
 static cudaError_t launch_line_kernel(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s,
                                       int cluster = 0)
 {
+    const cudaError_t e = allow_smem(kern, smem);
+    if (e != cudaSuccess) return e;
     return launch_kernel(kern, dim3((unsigned)nblocks), dim3((unsigned)nthreads), smem, s, a.chained != 0, cluster, a);
 }
 

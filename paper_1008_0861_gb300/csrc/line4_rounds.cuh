@@ -6,21 +6,6 @@
 
 namespace aniso {
 
-template <typename K>
-static cudaError_t run_rounds(K kern, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
-{
-    if (smem > 47 * 1024) {  // static shared memory counts against the 48 KB default
-        cudaFuncAttributes fa;
-        cudaError_t e = cudaFuncGetAttributes(&fa, kern);
-        if (e != cudaSuccess) return e;
-        if ((size_t)fa.maxDynamicSharedSizeBytes < smem &&
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-                cudaSuccess)
-            return e;
-    }
-    return launch_line_kernel(kern, a, nblocks, nthreads, smem, s);
-}
-
 template <template <int> class F>
 static cudaError_t by_rounds(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
 {

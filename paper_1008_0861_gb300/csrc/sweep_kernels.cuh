@@ -50,6 +50,19 @@ __device__ __forceinline__ void chain_wait()
 // and loads taken early hold registers from there on (256^3 FP32 3-D, 4 steps
 // 1135 us, 1165 without; 1024^2, 20 steps 340 and 344).
 template <typename T> __device__ __forceinline__ void after_wait(const T *&p) { asm volatile("" : "+l"(p)); }
+// Host: lets kern be launched with smem bytes of dynamic shared memory.  What is
+// above the default 48 KB (its static shared memory included) is allowed once, all
+// of it: a limit of this launch's size could be set between another thread's
+// look at the limit and its launch with more.
+template <typename K> static cudaError_t allow_smem(K kern, size_t smem)
+{
+    if (smem <= 47 * 1024) return cudaSuccess;
+    cudaFuncAttributes fa;
+    const cudaError_t e = cudaFuncGetAttributes(&fa, kern);
+    if (e != cudaSuccess || (size_t)fa.maxDynamicSharedSizeBytes >= smem) return e;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(SMEM_LIMIT - fa.sharedSizeBytes));
+}
 // Host: a launch of kern(a...), chained or plain, in clusters of `cluster` blocks (0: none).
 template <typename... P, typename... A>
 static cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool chained,
