@@ -84,8 +84,12 @@ enum {
                                  1: block-synchronous vectorised line kernel;
                                  0: general kernels only; 2 is not a valid value */
     ANISO_OPT_SEGMENT = 9,    /* cells per thread segment of the vectorised kernels, in 16-byte
-                                 chunks (0 = default: 4, fewer for a small FP64 grid stepped alone;
-                                 larger: fewer threads per line and so a shallower PCR) */
+                                 chunks (0 = default: 4; 1 for FP32 updates of at most 608 lines that
+                                 are ragged, see aniso_step, alone and in batches; fewer than 4 for a
+                                 small FP64 grid stepped alone; larger: fewer threads per line and so
+                                 a shallower PCR).  Segments decide the last bits: with a value of its
+                                 own here, 4 say, a small FP64 grid has the same bits alone as in a
+                                 batch whose first handle has that value or none. */
     ANISO_OPT_BLOCK_WARPS = 10, /* warps per block of the warp-autonomous kernel (0 = default: 4, 8 for
                                    middling FP32 grids stepped alone;
                                    1, 2, 4 or 8): lines per block = warps x lines per warp */
@@ -196,6 +200,11 @@ int aniso_set_source(aniso_t h, const void *Q);
  * The update order of each step follows ANISO_OPT_ORDER; the handle's step
  * counter (used by ANISO_ORDER_ALTERNATE) advances by nsteps.  With
  * ANISO_OPT_KAHAN the handle keeps the low parts of T between calls.
+ * Any side and any alignment of T to its element runs; the fastest kernels
+ * take sides that are multiples of the 16-byte vector (4 cells in FP32, 2 in
+ * FP64) and a T on a 16-byte boundary.  Others are ragged: lines up to 2048
+ * cells (FP32; 1024 in FP64) run in a form of the same kernel that loads cell
+ * by cell, for which the handle keeps transposed copies of the y coefficients.
  * Asynchronous.  Errors: ANISO_ERR_ARG, ANISO_ERR_STATE (no field),
  * ANISO_ERR_CUDA, ANISO_ERR_UNSUPPORTED (a line longer than the on-chip
  * limit: 16384 cells in FP32, 8192 in FP64). */
@@ -243,8 +252,8 @@ const char *aniso_last_error(void);
 
 /* Group n handles (same precision, limiter and field storage; each with its
  * field set) so that each sweep advances all of them together: one launch per
- * class of line lengths with the same occupancy (at most five, run
- * concurrently), the paper's update applied to independent grids of uneven
+ * class of line lengths with the same form and occupancy (at most nine of the
+ * warp-per-line kernel, run concurrently up to seven), the paper's update applied to independent grids of uneven
  * sizes, fields and timesteps.  The batch uses the first handle's stream and options
  * GRAPH/PROFILE.  The handles must outlive the batch.  Grids with more than
  * 1024 rows take their y-updates through the transpose path, captured into the
@@ -255,7 +264,8 @@ int aniso_batch_create(int n, const aniso_t *hs, aniso_batch_t *out);
  * T[k] (host arrays of n entries; T[k] a device pointer).  Grids with fewer
  * steps drop out as they finish.  The whole call is captured once into a
  * CUDA graph and replayed while T, dt and nsteps stay the same.
- * Asynchronous. */
+ * A grid has the same bits as with aniso_step, FP64 grids where their segments
+ * are the same (ANISO_OPT_SEGMENT).  Asynchronous. */
 int aniso_step_batched(aniso_batch_t b, void *const *T, const double *dt, const int *nsteps);
 
 /* aniso_step_batched on host arrays: T_host[k] is a host array of grid k's
@@ -278,7 +288,9 @@ int aniso_step_batched_host(aniso_batch_t b, void *const *T_host, const double *
  * finished by one small kernel per launch, so the call stays one graph.
  * Slots of steps a grid does not take, and of grids whose y-update does not
  * run on the warp-per-line kernel (off the fast path, columns above 2048
- * cells, or on the cluster kernel of ANISO_OPT_CLUSTER_LINES), are NaN.
+ * cells, or on the cluster kernel of ANISO_OPT_CLUSTER_LINES) or runs in its
+ * ragged form (a side that is no multiple of the 16-byte vector, T off a
+ * 16-byte boundary), are NaN.
  * *steps (may be NULL) receives the steps per grid (the call's largest
  * nsteps); out may be NULL to query it.  capacity: doubles available at out.
  * Synchronises the batch's stream.  Errors: ANISO_ERR_ARG (capacity),

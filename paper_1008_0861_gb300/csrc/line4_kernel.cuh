@@ -247,7 +247,8 @@ template <> struct Limit<double, true, true> {
 };
 
 // Which product of a flux is fused with the sum is spelled out, so that every
-// form of the kernel rounds alike (a batch equals its grids one by one).
+// form of the kernel rounds alike (a batch equals its grids one by one where
+// their segments are the same: always in FP32, with ANISO_OPT_SEGMENT in FP64).
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }

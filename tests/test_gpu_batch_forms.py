@@ -65,3 +65,26 @@ def test_a_first_grid_with_long_segments_takes_any_other(lib, prec, shape, offse
         lib.aniso_batch_destroy(b)
         a.close()
         g.close()
+
+
+@pytest.mark.parametrize("limiter", [0, 2])
+def test_fp64_grids_of_one_segment_length_have_the_same_bits_alone_and_in_a_batch(lib, limiter):
+    """A small FP64 grid alone takes shorter segments than in a batch; with the
+    default of 4 chunks asked for on the handle it takes the batch's."""
+    import torch
+    shapes = [(50, 50), (24, 24), (33, 47), (64, 200), (128, 96), (101, 67), (300, 40), (512, 512), (1100, 64)]
+    insts = [W.random_instance(*s, seed=k, dt_factor=20.0) for k, s in enumerate(shapes)]
+    grids = [GpuGrid(lib, i, FP64, limiter=limiter) for i in insts]
+    singles = [GpuGrid(lib, i, FP64, limiter=limiter) for i in insts]
+    for s in singles:
+        lib.aniso_set_option(s.h, lib.ANISO_OPT_SEGMENT, 4)
+    b = lib.aniso_batch_create([g.h for g in grids])
+    try:
+        lib.aniso_step_batched(b, [g.T for g in grids], [i.dt for i in insts], [4] * len(insts))
+        torch.cuda.synchronize()
+        for g, s in zip(grids, singles):
+            assert np.array_equal(g.T.cpu().numpy(), s.step(4))
+    finally:
+        lib.aniso_batch_destroy(b)
+        for g in grids + singles:
+            g.close()
