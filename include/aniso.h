@@ -87,9 +87,9 @@ enum {
                                  chunks (0 = default: 4; 1 for FP32 updates of at most 608 lines that
                                  are ragged, see aniso_step, alone and in batches; fewer than 4 for a
                                  small FP64 grid stepped alone; larger: fewer threads per line and so
-                                 a shallower PCR).  Segments decide the last bits: with a value of its
-                                 own here, 4 say, a small FP64 grid has the same bits alone as in a
-                                 batch whose first handle has that value or none. */
+                                 a shallower PCR).  Segments decide the last bits: with 4 here a
+                                 small FP64 grid has the same bits alone as in a batch, which takes
+                                 its value (default 4 in FP64) from its first handle. */
     ANISO_OPT_BLOCK_WARPS = 10, /* warps per block of the warp-autonomous kernel (0 = default: 4, 8 for
                                    middling FP32 grids stepped alone;
                                    1, 2, 4 or 8): lines per block = warps x lines per warp */
@@ -253,9 +253,9 @@ const char *aniso_last_error(void);
 /* Group n handles (same precision, limiter and field storage; each with its
  * field set) so that each sweep advances all of them together: one launch per
  * class of line lengths with the same form and occupancy (at most nine of the
- * warp-per-line kernel, run concurrently up to seven), the paper's update applied to independent grids of uneven
- * sizes, fields and timesteps.  The batch uses the first handle's stream and options
- * GRAPH/PROFILE.  The handles must outlive the batch.  Grids with more than
+ * warp-per-line kernel, up to seven at a time), the paper's update applied to
+ * independent grids of uneven sizes, fields and timesteps.  The batch uses the
+ * first handle's stream and options GRAPH/PROFILE.  The handles must outlive the batch.  Grids with more than
  * 1024 rows take their y-updates through the transpose path, captured into the
  * same graph.  Errors: ANISO_ERR_ARG, ANISO_ERR_STATE. */
 int aniso_batch_create(int n, const aniso_t *hs, aniso_batch_t *out);
