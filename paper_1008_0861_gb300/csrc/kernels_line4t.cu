@@ -1,5 +1,6 @@
 // Instantiations of the warp-per-line kernel's tensor-memory form with the
-// chunk rounds as a constant (VC), FP32 van Leer.
+// chunk rounds as a constant (VC), FP32 van Leer, 4 to 7 rounds (8 spilled: such
+// lines keep the run-time form).
 #include "line4_rounds.cuh"
 
 namespace aniso {
@@ -17,7 +18,7 @@ template <int VC> struct Tensor {
 cudaError_t launch_line4_rounds_tm(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem,
                                    cudaStream_t s)
 {
-    return by_rounds<Tensor>(coef_fp16, a, nblocks, nthreads, smem, s);
+    return by_rounds<Tensor, 7>(coef_fp16, a, nblocks, nthreads, smem, s);
 }
 
 }  // namespace aniso

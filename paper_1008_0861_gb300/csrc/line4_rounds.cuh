@@ -6,7 +6,7 @@
 
 namespace aniso {
 
-template <template <int> class F>
+template <template <int> class F, int LAST = 8>
 static cudaError_t by_rounds(int coef_fp16, const Line2Args &a, int nblocks, int nthreads, size_t smem, cudaStream_t s)
 {
     switch (a.rounds) {
@@ -14,7 +14,9 @@ static cudaError_t by_rounds(int coef_fp16, const Line2Args &a, int nblocks, int
     case 5: return F<5>::run(coef_fp16, a, nblocks, nthreads, smem, s);
     case 6: return F<6>::run(coef_fp16, a, nblocks, nthreads, smem, s);
     case 7: return F<7>::run(coef_fp16, a, nblocks, nthreads, smem, s);
-    case 8: return F<8>::run(coef_fp16, a, nblocks, nthreads, smem, s);
+    case 8:
+        if constexpr (LAST == 8) return F<8>::run(coef_fp16, a, nblocks, nthreads, smem, s);
+        else return cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
 }
