@@ -28,7 +28,8 @@
 // (Line2Job::swz, line4_swizzle) for the segment lengths it has, the default
 // being log2 of the chunks per segment.
 // FP32 reciprocals use the hardware approximation (rcp.approx.ftz.f32,
-// within 1 ulp); FP64 divides exactly.  Each block first asks for its input
+// within 1 ulp); FP64 quotients are rounded but for rare neighbours (dquot).
+// Each block first asks for its input
 // rows to be brought into L2 with bulk prefetches.
 //
 // D3: the lines of a three-dimensional grid (Section 2.1).  The face flux
