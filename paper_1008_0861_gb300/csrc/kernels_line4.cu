@@ -163,12 +163,12 @@ bool line4_chain(int nblocks, size_t smem)
 // its group of 8 chunks (the last, incomplete group unswizzled).  The
 // coalesced phases have the 8 lanes of a quarter warp touch one whole group,
 // conflict-free under any such permutation.  The segment phases have lane t
-// walk chunks c_lo(t) + u of its segment (U + 1 chunks for the first m mod P
-// lanes, U for the rest), so a quarter warp's chunks lie a segment length
-// apart and their bank groups (chunk mod 8) repeat unless the shift spreads
-// them.  Each candidate (log2 U, none, 1..6) is scored by the wavefronts of
+// walk chunks ce(t) - k from its segment's last down (U + 1 chunks for the first
+// m mod P lanes, U for the rest) and back up, so a quarter warp's chunks lie a
+// segment length apart and their bank groups (chunk mod 8) repeat unless the
+// shift spreads them.  Each candidate (log2 U, none, 1..6) is scored by the wavefronts of
 // those walks, the largest number of a quarter's lanes on one bank group,
-// summed over the steps u and the quarters; the first lowest wins.
+// summed over the steps k and the quarters; the first lowest wins.
 int line4_swizzle(int prec, int n, int team)
 {
     const int N = prec == PREC_FP64 ? 2 : 4;
@@ -183,12 +183,13 @@ int line4_swizzle(int prec, int n, int team)
     for (int code = 0; code <= 7; ++code) {
         const int sh = code >= 2 ? code - 1 : logU, msk = code == 1 ? 0 : 7;
         long w = 0;
-        for (int u = 0; u < V; ++u)
+        for (int k = 0; k < V; ++k)
             for (int q0 = 0; q0 < P; q0 += 8) {
                 int cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
                 for (int t = q0; t < q0 + 8; ++t) {
-                    if (u >= U + (t < rr ? 1 : 0)) continue;
-                    const int c = t * U + (t < rr ? t : rr) + u;
+                    const int Ut = U + (t < rr ? 1 : 0);
+                    if (k >= Ut) continue;
+                    const int c = t * U + (t < rr ? t : rr) + Ut - 1 - k;
                     ++cnt[(c < mfull ? c ^ ((c >> sh) & msk) : c) & 7];
                 }
                 int mx = 0;
