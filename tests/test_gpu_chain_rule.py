@@ -38,3 +38,31 @@ def test_chained_calls_keep_the_chip_evenly_filled(lib, nx, ny, prec, order):
     finally:
         a.close()
         b.close()
+
+
+@pytest.mark.parametrize("n", [(32, 32, 32), (20, 64, 36), (64, 64, 64), (96, 100, 104), (136, 192, 60)])
+@pytest.mark.parametrize("prec,fp16", [(FP32, False), (FP32, True), (FP64, False)])
+@pytest.mark.parametrize("scheme", [0, 1])
+def test_3d_steps_of_one_call_equal_steps_waited_for(lib, n, prec, fp16, scheme):
+    """Within a call the launches overlap and ask for other amounts of shared
+    memory; one-step calls with a wait after each keep all but two apart."""
+    import torch
+    inst = W.random_instance3d(*n, seed=3)
+    dt = torch.float64 if prec == FP64 else torch.float32
+    got = []
+    for calls, steps in ((1, 6), (6, 1)):
+        h = lib.aniso3_create(*n, inst.dx, inst.dy, inst.dz, inst.chi_par, 0.0, inst.bc)
+        try:
+            lib.aniso3_set_option(h, lib.ANISO_OPT_PRECISION, prec)
+            lib.aniso3_set_option(h, lib.ANISO_OPT_FIELD_FP16, int(fp16))
+            lib.aniso3_set_option(h, lib.ANISO_OPT_SCHEME, scheme)
+            lib.aniso3_set_field(h, *(torch.tensor(v, dtype=dt, device="cuda") for v in (inst.bx, inst.by, inst.bz)))
+            T = torch.tensor(inst.T0, dtype=dt, device="cuda")
+            for _ in range(calls):
+                lib.aniso3_step(h, T, inst.dt, steps)
+                torch.cuda.synchronize()
+            lib.aniso3_sync(h)
+            got.append(T)
+        finally:
+            lib.aniso3_destroy(h)
+    assert torch.equal(*got)
