@@ -259,6 +259,11 @@ __device__ __forceinline__ double fma_rn(double a, double b, double c) { return 
 __device__ __forceinline__ bool non_finite(float v) { return !(fabsf(v) < INFINITY); }
 __device__ __forceinline__ bool non_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 
+// p + 0 v: p = 0 stays 0 while every v is finite and is NaN from the first that is
+// not.  FP32: one test a lane at the end instead of one a chunk on its sum, which
+// can leave the range where its values do not.
+__device__ __forceinline__ float finite_probe(float p, float v) { return __fmaf_rn(v, 0.f, p); }
+
 // PCR over a team of P <= 32 lanes (width-P shuffles), as pcr_warp.  Each lane
 // takes the reciprocal of its own diagonal once and hands that on, instead of
 // dividing by both neighbours' diagonals (the quotients' bits are kept).
@@ -873,6 +878,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
 
     // ---- C: T_new = T_old + delta, coalesced
     bool bad = false;
+    R probe = R(0);
     // diagnostics: compensated sum of the chunk sums, min, max of this lane's cells
     const bool diag = args.diag_part != nullptr;
     R dh = R(0), dl = R(0), dmn = R(INFINITY), dmx = R(-INFINITY);
@@ -892,16 +898,16 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
                 if (c + 2 * P < m) pre1 = ld_old(c + 2 * P);
             }
             V16<R>::unpack(sA[swz(c)], d);
-            R sum = R(0);
 #pragma unroll
             for (int j = 0; j < N; ++j) {
                 to[j] += d[j];
-                if constexpr (N == 4) sum += to[j];  // FP32: one test for the chunk
+                if constexpr (N == 4) probe = finite_probe(probe, to[j]);
                 else bad |= non_finite(to[j]);
             }
-            if constexpr (N == 4) bad |= non_finite(sum);
             if (diag && active) {
-                if constexpr (N != 4) sum = to[0] + to[1];
+                R sum = R(0);
+#pragma unroll
+                for (int j = 0; j < N; ++j) sum += to[j];
                 const R y = sum - dl, tt = dh + y;
                 dl = (tt - dh) - y;
                 dh = tt;
@@ -962,7 +968,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 && RING == 1 ? (D3 ? 3 : 4
             }
         }
     }
-    if (bad && active) atomicOr(args.err, 1u);
+    if ((bad || (N == 4 && non_finite(probe))) && active) atomicOr(args.err, 1u);
     if (diag) {  // the block's partial, reduced in a fixed order (deterministic)
         __shared__ DiagPart s_diag[8];
         double ds = (double)dh - (double)dl, mn = (double)dmn, mx = (double)dmx;

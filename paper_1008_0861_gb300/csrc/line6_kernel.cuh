@@ -283,6 +283,7 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
 
     // ---- C: T_new = T_old + delta, coalesced; staged for the store
     bool bad = false;
+    R probe = R(0);
     for (int v = 0; v < V; ++v) {
         const int c = v * P + t;
         if (c >= m) break;
@@ -291,14 +292,12 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
         pre0 = pre1;
         if (c + 2 * P < m) pre1 = vcC[c + 2 * P];
         V16<R>::unpack(sA[swz(c)], d);
-        R sum = R(0);
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             to[j] += d[j];
-            if constexpr (N == 4) sum += to[j];
+            if constexpr (N == 4) probe = finite_probe(probe, to[j]);
             else bad |= non_finite(to[j]);
         }
-        if constexpr (N == 4) bad |= non_finite(sum);
         if (!J.transpose_out) {
             if (active) reinterpret_cast<VT *>(static_cast<R *>(J.Tout) + (size_t)lc * n)[c] = V16<R>::pack(to);
         } else {
@@ -349,7 +348,7 @@ __global__ void __launch_bounds__(512, 1) line6_kernel(Line2Args args)
             }
         }
     }
-    if (bad && active) atomicOr(args.err, 1u);
+    if ((bad || (N == 4 && non_finite(probe))) && active) atomicOr(args.err, 1u);
 }
 
 }  // namespace aniso

@@ -623,7 +623,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
     }
 
     // ---- C: T_new = T_old + delta, coalesced; staged for the store
-    bool bad = false;
+    R probe = R(0);
 #pragma unroll
     for (int v = 0; v < V; ++v) {
         const int c = v * P + t;
@@ -643,7 +643,6 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
         }
         V16<R>::unpack(sA[cz(v)], d);
         R hi[N], lo[N];
-        R sum = R(0);
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             if (K) {
@@ -652,9 +651,8 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
                 hi[j] = to[j] + d[j];
                 lo[j] = R(0);
             }
-            sum += hi[j];
+            probe = finite_probe(probe, hi[j]);
         }
-        bad |= !(fabsf(sum) < INFINITY);
         if (!J.transpose_out) {
             if (active && ilv_out) {
                 VT *o = reinterpret_cast<VT *>(static_cast<R *>(J.Tout) + (size_t)lc * 2 * n) + 2 * (q0 + c);
@@ -744,7 +742,7 @@ __global__ void __launch_bounds__(L7_THREADS, TM ? 3 : 2) line7_kernel(Line2Args
             }
         }
     }
-    if (bad && active) atomicOr(args.err, 1u);
+    if (non_finite(probe) && active) atomicOr(args.err, 1u);
     if (TO) {  // every warp is done with TMEM before the block frees it
         tm_fence_before();
         __syncthreads();
