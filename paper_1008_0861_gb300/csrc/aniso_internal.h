@@ -228,9 +228,9 @@ int line4_warps_alone(int n, int nlines);
 // dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each, and whether the launch may be
 // chained with it.
 size_t line4_smem_alone(int nblocks, size_t smem);
+bool line4_chain(int nblocks, size_t smem);
 // whether an FP32 launch alone takes the form with three rounds of loads in flight.
 bool line4_deep(int nblocks, int nthreads);
-bool line4_chain(int nblocks, size_t smem);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.
 int line4_tm_cols(int n, int team);
 // Chunks of padding after each warp's shared area in the FP32 line4 kernel

@@ -29,8 +29,8 @@
 // being log2 of the chunks per segment.
 // FP32 reciprocals use the hardware approximation (rcp.approx.ftz.f32,
 // within 1 ulp); FP64 quotients are rounded but for rare neighbours (dquot).
-// Each block first asks for its input
-// rows to be brought into L2 with bulk prefetches.
+// Each block first asks for its input rows to be brought into L2 with bulk
+// prefetches.
 //
 // D3: the lines of a three-dimensional grid (Section 2.1).  The face flux
 // gains a second limited transverse term, mu2 * e2 * DeltaT-bar along the
