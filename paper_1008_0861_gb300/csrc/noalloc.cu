@@ -187,7 +187,7 @@ extern "C" int aniso_step_noalloc(int nx, int ny, double dx, double dy, double c
 
     // Both updates on the warp-per-line kernel (x: rows of T to a column-major
     // T*; y: T*'s columns back to rows of T), wherever it takes lines of these
-    // lengths: 96 x 64 FP32, one step 23.3 us on the general kernels, 10.2 here.
+    // lengths: 96 x 64 FP32, one step 23.2 us on the general kernels, 11.3 here.
     LineLaunch lx, ly;
     if (line_launch(precision, nx, ny, T, tstar, cxx, cxy, lamx, mu, per, err, &lx) &&
         line_launch(precision, ny, nx, tstar, T, cyy, cyx, lamy, mu, per, err, &ly)) {
