@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -1251,6 +1252,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
     // classes of a sweep run concurrently (one graph branch each).
     int shape_rc = ANISO_OK;
     int next_group = 0;
+    std::map<std::pair<int, int>, int> swizzles;  // (cells, team) -> shift
     auto add_line4 = [&](std::vector<Line2Job> &jobs, int kind_xy, int group) {
         if (jobs.empty()) return;
         const int warps = b->hs[0]->l4_warps, seg = b->hs[0]->seg_chunks;
@@ -1293,7 +1295,9 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                               ragged(J)) ||
                 nt != nthreads)
                 shape_rc = fail(ANISO_ERR_UNSUPPORTED, "batch: line length %d does not fit the block shape", J.n);
-            J.swz = line4_swizzle(prec, J.n, J.team);
+            const auto swz = swizzles.emplace(std::make_pair(J.n, J.team), 0);  // (counted once a length)
+            if (swz.second) swz.first->second = line4_swizzle(prec, J.n, J.team);
+            J.swz = swz.first->second;
             int occ = line4_blocks_per_sm(prec, fp16, b->hs[0]->limiter, nthreads, sm, false);
             const int rounds = ragged(J) ? 0 : line4_rounds(prec, b->hs[0]->limiter, J.n, J.team);
             cls[k] = {occ > 0 ? occ : 0, sm, ragged(J) ? 2 : 0, rounds};
@@ -1470,6 +1474,8 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
         }
         return true;
     };
+    std::vector<int> kinds(n);  // every grid's fast_kind for the call, 0: general
+    for (int k = 0; k < n; ++k) kinds[k] = on_fast_path(b->hs[k], T[k]) ? b->hs[k]->fast_kind() : 0;
     size_t step_begin = 0;
     for (int s = 0; s < max_steps; ++s) {
         for (int phase = 0; phase < 2; ++phase) {
@@ -1482,7 +1488,8 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
             for (int k = 0; k < n; ++k) {
                 if (s >= nsteps[k]) continue;
                 aniso_ctx *h = b->hs[k];
-                if (on_fast_path(h, T[k]) && h->fast_kind() == 7) {
+                const int fk = kinds[k];
+                if (fk == 7) {
                     // cluster-kernel grids (and the compensated state): the
                     // grid's fast update captured on its own
                     Launch L{13, 0, 0, 0, 0, 0};
@@ -1493,7 +1500,7 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                     solo.push_back(L);
                     continue;
                 }
-                if (on_fast_path(h, T[k])) {
+                if (fk != 0) {
                     // x: T (rows) -> T* (column-major); y: T* (columns) -> T (rows)
                     const int per = h->bc == ANISO_BC_PERIODIC;
                     const double mu = h->chi_par * dt[k] / (h->dx * h->dy);
@@ -1526,7 +1533,6 @@ static int batch_build(aniso_batch *b, void *const *T, const double *dt, const i
                         (diag && phase == 1 && h->whole_vectors() && aligned16(T[k])) ? k * max_steps + s : -1;
                     int t5, l5, n5;
                     size_t s5;
-                    const int fk = h->fast_kind();
                     if ((fk == 4 || fk == 6) && tma_mode && J.nlines % 4 == 0 && aligned16(J.Tin) &&
                         aligned16(J.Tout) && !(diag && phase == 1) && line5_available() &&
                         line5_config(prec, fp16, J.n, &t5, &l5, &n5, &s5)) {
