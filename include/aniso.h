@@ -72,7 +72,9 @@ enum {
     ANISO_OPT_KAHAN = 2,      /* 1: compensated FP32 state, T + lo (FP32 precision only) */
     ANISO_OPT_LIMITER = 3,    /* ANISO_LIM_* */
     ANISO_OPT_ORDER = 4,      /* ANISO_ORDER_* */
-    ANISO_OPT_STREAM = 5,     /* cudaStream_t cast to integer; 0 = legacy default stream */
+    ANISO_OPT_STREAM = 5,     /* cudaStream_t cast to integer; 0 = legacy default stream, on which a
+                                 step's launches may keep other streams' work out of the SMs they
+                                 use: a handle that runs beside other work belongs on its own */
     ANISO_OPT_GRAPH = 6,      /* 1 (default): replay aniso_step loops from a captured CUDA graph */
     ANISO_OPT_PROFILE = 7,    /* 1: time every sweep launch with CUDA events (aniso_kernel_times);
                                  k > 1: batched calls time the sweeps of every k-th step of a

@@ -204,10 +204,7 @@ static int enqueue3(aniso3_ctx *h, int d, const void *in, void *out, double lam,
     if (A.rounds > 5) A.rounds = 0;
     J.block0 = 0;
     J.nblocks = (J.nlines + J.lines_per_block - 1) / J.lines_per_block;
-    if (chained) {
-        smem = line4_smem_alone(J.nblocks, smem);
-        A.chained = line4_chain(J.nblocks, smem);
-    }
+    if (chained) A.chained = line4_chain(h->stream == 0, J.nblocks, &smem);
     CU(launch_line4_3d(h->prec, h->field_fp16, A, J.nblocks, nthreads, smem, h->stream));
     return ANISO_OK;
 }

@@ -464,10 +464,7 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     J.nblocks = (nlines + J.lines_per_block - 1) / J.lines_per_block;
     a.chained = h->chained && !h->profile && !v7;  // (a timing event between two launches keeps them apart)
     h->chained = true;
-    if (v4 && a.chained) {
-        smem = line4_smem_alone(J.nblocks, smem);
-        a.chained = line4_chain(J.nblocks, smem);
-    }
+    if (v4 && a.chained) a.chained = line4_chain(h->stream == 0, J.nblocks, &smem);
     int pidx = -1;
     const unsigned rec_flags = pairs ? cudaEventRecordExternal : cudaEventRecordDefault;
     if (h->profile) {

@@ -225,10 +225,9 @@ int line4_seg_fp64(int n, int nlines);
 int line4_seg_ragged(int nlines);
 // warps a block (0: the default) for an FP32 update of nlines lines of n cells launched alone.
 int line4_warps_alone(int n, int nlines);
-// dynamic shared memory for a chained launch of nblocks blocks that need smem bytes each, and whether the launch may be
-// chained with it.
-size_t line4_smem_alone(int nblocks, size_t smem);
-bool line4_chain(int nblocks, size_t smem);
+// whether a launch of nblocks blocks that need *smem bytes each may be chained on the legacy default stream, or on
+// another one; raises *smem where that takes more.
+bool line4_chain(bool default_stream, int nblocks, size_t *smem);
 // whether an FP32 launch alone takes the form with three rounds of loads in flight.
 bool line4_deep(int nblocks, int nthreads);
 // TMEM columns a line4 block of lines of n cells (teams of `team` lanes) allocates.

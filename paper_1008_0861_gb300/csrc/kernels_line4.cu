@@ -134,29 +134,29 @@ int line4_warps_alone(int n, int nlines)
     return blocks >= 96 && blocks <= 152 * (resident < 4 ? resident : 4) ? 8 : 0;
 }
 
-// Dynamic shared memory for a chained launch: enough that an SM holds no more
-// than its share of the blocks.  A chained launch's blocks are placed while their
-// predecessor drains, on whichever SMs are free first, and with room for more one
-// SM gets several of them and another none, which then lasts for the whole launch.
-// us, unchained / with the natural size / with this one: FP64 352 x 512, 20 steps
-// 1218 / 2762 / 1184; FP32 777 x 1001, 20 steps 533 / 754 / 518; FP32 512^2 4-step
-// 358 / 465 / 329; FP32 1024^2 an update 9.6 / 9.7 / 9.0; 3-D FP32 136 x 192 x 60,
-// 3 steps 160 / 201 / 141.
-size_t line4_smem_alone(int nblocks, size_t smem)
+// Whether a launch of nblocks blocks that need *smem bytes of dynamic shared
+// memory each may be chained, with *smem raised where that takes more.  A chained
+// launch's blocks are placed while their predecessor drains, on whichever SMs are
+// free first, and with room for more than its share of the blocks one SM gets
+// several of them and another none, which then lasts for the whole launch.  So
+// each block asks for as much as keeps an SM to its share.  us, unchained / with
+// the natural size / with this one: FP64 352 x 512, 20 steps 1218 / 2762 / 1184; FP32
+// 777 x 1001, 20 steps 533 / 754 / 518; FP32 512^2 4-step 358 / 465 / 329; FP32 1024^2
+// an update 9.6 / 9.7 / 9.0; 3-D FP32 136 x 192 x 60, 3 steps 160 / 201 / 141.
+// That shuts other streams' blocks out of the SM (8 handles of 512^2 FP32 on 8
+// streams, 20 steps: 447 us unchained, 978 with it).  It is done on the legacy
+// default stream alone, whose work is not shared with other blocking streams; on a
+// stream of the caller's only launches of at most 76 blocks are chained, which fit
+// the chip beside the launch before, with their natural size (16 handles of 300^2,
+// 40 steps: 764 us unchained, 551 so, 1468 with the raised one).
+bool line4_chain(bool default_stream, int nblocks, size_t *smem)
 {
+    const bool few = nblocks <= 76;
+    if (!default_stream) return few;
     const int share = (nblocks + 151) / 152;
-    if (share > 4) return smem;
-    const size_t least = (size_t)228 * 1024 / (share + 1) - 1024 + 16;
-    return smem > least ? smem : least;
-}
-
-// Whether a launch of nblocks blocks with smem bytes each may be chained: an SM
-// has room for its share of them and no more (above), or they are so few that
-// they fit the chip beside the launch before.
-bool line4_chain(int nblocks, size_t smem)
-{
-    const int share = (nblocks + 151) / 152, room = (int)((size_t)228 * 1024 / (smem + 1024));
-    return nblocks <= 76 || room <= share;
+    const size_t sm = (size_t)228 * 1024, least = sm / (share + 1) - 1024 + 16;
+    if (share <= 4 && *smem < least) *smem = least;
+    return few || (int)(sm / (*smem + 1024)) <= share;
 }
 
 // The kernel keeps 16-byte chunk c of a line at c ^ ((c >> s) & 7) inside

@@ -107,7 +107,7 @@ struct LineLaunch {
 
 // False when the kernel does not take lines of n cells.
 bool line_launch(int prec, int n, int nlines, const void *in, void *out, const void *g, const void *e, double lam,
-                 double mu, int per, unsigned *err, LineLaunch *L)
+                 double mu, int per, unsigned *err, bool default_stream, LineLaunch *L)
 {
     const int vec = prec == PREC_FP64 ? 2 : 4;
     auto off = [](const void *p) { return ((uintptr_t)p & 15) != 0; };
@@ -135,8 +135,7 @@ bool line_launch(int prec, int n, int nlines, const void *in, void *out, const v
     J.swz = line4_swizzle(prec, n, J.team);
     L->args.rounds = L->ragged ? 0 : line4_rounds(prec, LIM_VANLEER, n, J.team);
     J.nblocks = (nlines + J.lines_per_block - 1) / J.lines_per_block;
-    L->smem = line4_smem_alone(J.nblocks, L->smem);
-    L->args.chained = line4_chain(J.nblocks, L->smem);
+    L->args.chained = line4_chain(default_stream, J.nblocks, &L->smem);
     return true;
 }
 
@@ -189,8 +188,8 @@ extern "C" int aniso_step_noalloc(int nx, int ny, double dx, double dy, double c
     // T*; y: T*'s columns back to rows of T), wherever it takes lines of these
     // lengths: 96 x 64 FP32, one step 23.2 us on the general kernels, 11.3 here.
     LineLaunch lx, ly;
-    if (line_launch(precision, nx, ny, T, tstar, cxx, cxy, lamx, mu, per, err, &lx) &&
-        line_launch(precision, ny, nx, tstar, T, cyy, cyx, lamy, mu, per, err, &ly)) {
+    if (line_launch(precision, nx, ny, T, tstar, cxx, cxy, lamx, mu, per, err, s == 0, &lx) &&
+        line_launch(precision, ny, nx, tstar, T, cyy, cyx, lamy, mu, per, err, s == 0, &ly)) {
         e = launch_face_coeffs(precision, coef, bx, by, nx, ny, bc, kappa, cxx, cxy, nullptr, nullptr, cyy, cyx, s);
         LineLaunch first = lx;
         first.after_coeffs(precision);

@@ -66,3 +66,31 @@ def test_3d_steps_of_one_call_equal_steps_waited_for(lib, n, prec, fp16, scheme)
         finally:
             lib.aniso3_destroy(h)
     assert torch.equal(*got)
+
+
+@pytest.mark.parametrize("n,handles,most", [(512, 8, 4.0), (1024, 4, 3.0), (300, 16, 3.0)])
+def test_handles_on_streams_of_their_own_share_the_gpu(lib, n, handles, most):
+    """Several handles stepped at once, each on its own stream, against one of
+    them alone: 1.7, 1.9 and 1.4 times as long with every launch plain; 6.4, 3.8
+    and 4.4 where chained blocks kept an SM to themselves."""
+    import torch
+    insts = [W.random_instance(n, n, seed=k, dt_factor=20.0) for k in range(handles)]
+    grids = [GpuGrid(lib, i, FP32) for i in insts]
+    streams = [torch.cuda.Stream() for _ in insts]
+    try:
+        torch.cuda.synchronize()
+        for g, s in zip(grids, streams):
+            lib.aniso_set_option(g.h, lib.ANISO_OPT_STREAM, s.cuda_stream)
+
+        def run(some):
+            for _ in range(4):
+                for g, i in some:
+                    lib.aniso_step(g.h, g.T, i.dt, 20)
+
+        pairs = list(zip(grids, insts))
+        alone, all_at_once = (_best(lambda some=some: run(some), 9) for some in (pairs[:1], pairs))
+        assert all_at_once < most * alone
+    finally:
+        torch.cuda.synchronize()
+        for g in grids:
+            g.close()
