@@ -403,6 +403,7 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
     a.njobs = 1;
     a.limiter = h->limiter;
     a.err = h->err;
+    a.shared = h->stream != 0;
     Line2Job &J = a.one;
     J.Tin = in;
     J.Tout = out;
@@ -430,7 +431,7 @@ static int enqueue_line2(aniso_ctx *h, const void *in, void *out, const void *g,
                     : h->prec == PREC_FP64 ? line4_seg_fp64(n, nlines)
                     : ragged               ? line4_seg_ragged(nlines)
                                            : 0;
-    const int warps = v4 && transposed && h->l4_warps == 0 && h->seg_chunks == 0 && h->prec == PREC_FP32
+    const int warps = v4 && transposed && !a.shared && h->l4_warps == 0 && h->seg_chunks == 0 && h->prec == PREC_FP32
                           ? line4_warps_alone(n, nlines)
                           : h->l4_warps;
     bool ok = v4 ? line4_config(h->prec, n, transposed, warps, seg, &J.team, &J.lines_per_block, &nthreads,

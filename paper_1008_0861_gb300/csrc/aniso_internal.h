@@ -141,6 +141,8 @@ struct Line2Args {
     // are then read with plain loads (the read-only path is for data that does not
     // change while a kernel is resident)
     int fresh;
+    // line4, a grid alone: 1: on a stream of the caller's, perhaps beside others
+    int shared;
     // line4, FP32 van Leer: the chunk rounds of every line of the launch, 4 to 8
     // (line4_rounds), to run the form that has them as a constant; 0: any
     int rounds;

@@ -14,7 +14,9 @@ cudaError_t launch_line4(int prec, int coef_fp16, const Line2Args &a, int nblock
                          cudaStream_t s)
 {
     const bool vl = a.limiter == LIM_VANLEER;
-    const bool deep = !a.jobs && line4_deep(nblocks, nthreads);
+    // (with run-time rounds it spills, which shows where several streams fill the
+    // GPU: 4 handles of 1216^2 on 4 streams, 20 steps: 1495 us one round, 2030 three)
+    const bool deep = !a.jobs && line4_deep(nblocks, nthreads) && (!a.shared || a.rounds);
     if (a.fresh) {
         if (!vl || a.jobs || a.one.chi_alpha != 0.0 || coef_fp16 || (prec == PREC_FP32 && !deep)) return cudaErrorInvalidValue;
         if (prec == PREC_FP64)
@@ -124,7 +126,8 @@ int line4_seg_ragged(int nlines) { return nlines <= 608 ? 1 : 0; }
 // store writes half sectors; eight warps write whole ones.  That is taken where
 // eight-warp blocks fill most SMs and run in one wave (768^2: 7.55 -> 7.26 us an
 // update, 1024^2: 10.2 -> 9.4; 512^2, 64 blocks: 4.63 -> 5.37; 1280^2, a second
-// wave: 13.9 -> 20.4).
+// wave: 13.9 -> 20.4), and on the legacy default stream only: beside other streams'
+// work they lose (8 handles of 768^2 on 8 streams, 20 steps: 895 -> 920 us).
 int line4_warps_alone(int n, int nlines)
 {
     int team, lpb, nt;

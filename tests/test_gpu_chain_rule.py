@@ -68,11 +68,12 @@ def test_3d_steps_of_one_call_equal_steps_waited_for(lib, n, prec, fp16, scheme)
     assert torch.equal(*got)
 
 
-@pytest.mark.parametrize("n,handles,most", [(512, 8, 4.0), (1024, 4, 3.0), (300, 16, 3.0)])
+@pytest.mark.parametrize("n,handles,most", [(512, 8, 4.0), (1024, 4, 3.0), (300, 16, 3.0), (1216, 4, 3.4)])
 def test_handles_on_streams_of_their_own_share_the_gpu(lib, n, handles, most):
     """Several handles stepped at once, each on its own stream, against one of
-    them alone: 1.7, 1.9 and 1.4 times as long with every launch plain; 6.4, 3.8
-    and 4.4 where chained blocks kept an SM to themselves."""
+    them alone: 1.7, 1.9, 1.4 and 2.8 times as long with every launch plain; 6.4,
+    3.8 and 4.4 where chained blocks kept an SM to themselves, 4.1 (1216) with three
+    rounds of loads in flight."""
     import torch
     insts = [W.random_instance(n, n, seed=k, dt_factor=20.0) for k in range(handles)]
     grids = [GpuGrid(lib, i, FP32) for i in insts]
